@@ -199,7 +199,7 @@ const DeviceInfo& device_info() {
       d.ok = march_set_attributes() == cudaSuccess && march_set_attributes_l2() == cudaSuccess &&
              march_set_attributes_parked() == cudaSuccess &&
              batch_set_attributes() == cudaSuccess &&
-             setup_set_attributes() == cudaSuccess && pass3d_set_attributes() == cudaSuccess;
+             time_set_attributes() == cudaSuccess && pass3d_set_attributes() == cudaSuccess;
   }
   cache[dev] = d;
   return cache[dev];
@@ -255,6 +255,7 @@ struct bpm_plan_s {
   double* refl = nullptr;
   double* trans = nullptr;
   double2* eh_time = nullptr;
+  double2* time_tab = nullptr;   // tables of the frequency-to-time transform (null: direct sum)
   int* dflag = nullptr;
   double* u_tmp = nullptr;
   float* gcorr = nullptr;        // 3D: curvature factor per column
@@ -315,7 +316,7 @@ void free_plan_buffers(bpm_plan p) {
                   p->rev,    p->gain,    p->omega, p->weight, p->inc_norm, p->refl,
                   p->trans,  p->eh_time, p->dflag, p->u_tmp,  p->gcorr,    p->twy,
                   p->qy,     p->spec,    p->twx3,  p->twiddle_t, p->twiddle_p, p->mask,
-                  p->cspan};
+                  p->cspan,  p->time_tab};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->ev0) cudaEventDestroy(p->ev0);
@@ -391,7 +392,7 @@ size_t plan_bytes(const bpm_grid& g, int n_ch) {
   b += size_t(g.nx) * (sizeof(float2) + sizeof(int) + sizeof(double));
   if (g.dims == 2) b += 3 * size_t(g.nx) * sizeof(float2);  // thread-order twiddles, pairs
   b += size_t(n_ch) * (5 * sizeof(double) + sizeof(double2));
-  b += nf * sizeof(double2);                       // time response
+  b += (nf + time_table_elems(n_ch)) * sizeof(double2);  // time response, its transform's tables
   return b;
 }
 
@@ -491,6 +492,7 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
   check(dalloc(&p->refl, size_t(n_channels)), "alloc R");
   check(dalloc(&p->trans, size_t(n_channels)), "alloc T");
   check(dalloc(&p->eh_time, nf), "alloc time response");
+  check(dalloc(&p->time_tab, time_table_elems(n_channels)), "alloc time tables");
   check(dalloc(&p->dflag, size_t(4)), "alloc status");
   if (g.dims == 3) {
     check(dalloc(&p->gcorr, size_t(n_channels) * 2 * g.nx), "alloc curvature factors");
@@ -527,6 +529,7 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
                         p->stream),
         "upload gain");
   check(cudaMemsetAsync(p->dflag, 0, sizeof(int) * 4, p->stream), "clear status");
+  check(launch_time_tables(n_channels, p->time_tab, p->stream), "time tables");
   std::vector<float2> qyt;
   if (g.dims == 3) {
     const FftConsts& fy = fft_consts(g.ny);
@@ -728,12 +731,25 @@ BPM_API bpm_status bpm_set_channel_shard(bpm_plan p, int first, int n_total, dou
     return fail(p, BPM_ERR_INVALID_ARG, "d_omega must be positive and finite");
   if (p->z != 0) return fail(p, BPM_ERR_STATE, "set the shard before the march starts");
   const int rows = std::max(p->shard_total, p->n_ch);
-  if (n_total > rows) {
-    double2* t = nullptr;
-    BPM_CUDA(p, dalloc(&t, size_t(n_total) * p->plane), "alloc time response");
-    cudaFree(p->eh_time);
-    p->eh_time = t;
-    p->bytes += size_t(n_total - rows) * p->plane * sizeof(double2);
+  if (n_total != time_rows(p)) {
+    double2 *t = nullptr, *tab = nullptr;
+    if (n_total > rows) BPM_CUDA(p, dalloc(&t, size_t(n_total) * p->plane), "alloc time response");
+    cudaError_t e = dalloc(&tab, time_table_elems(n_total));
+    if (e == cudaSuccess) e = launch_time_tables(n_total, tab, p->stream);
+    if (e != cudaSuccess) {
+      cudaFree(t);
+      cudaFree(tab);
+      BPM_CUDA(p, e, "time tables");
+    }
+    if (t) {
+      cudaFree(p->eh_time);
+      p->eh_time = t;
+      p->bytes += size_t(n_total - rows) * p->plane * sizeof(double2);
+    }
+    cudaFree(p->time_tab);
+    p->time_tab = tab;
+    p->bytes += time_table_elems(n_total) * sizeof(double2);
+    p->bytes -= time_table_elems(time_rows(p)) * sizeof(double2);
   }
   p->sharded = true;
   p->shard_first = first;
@@ -842,7 +858,7 @@ BPM_API bpm_status bpm_run(bpm_plan p, int n_steps) {
   p->time_valid = false;
   if (p->z == p->grid.nz) {
     BPM_CUDA(p, launch_omega_to_t(time_rows(p), p->shard_first, p->n_ch, p->plane, p->domega,
-                                  p->eh, p->eh_time, p->stream),
+                                  p->time_tab, p->eh, p->eh_time, p->stream),
              "omega-to-t kernel");
     ++launches;
     p->time_valid = true;
@@ -1370,7 +1386,7 @@ bpm_status enqueue_round(bpm_batch b, RoundSlot& r, int chunk) {
     p->time_valid = false;
     if (p->z == p->grid.nz) {
       BPM_BCUDA(b, launch_omega_to_t(time_rows(p), p->shard_first, p->n_ch, p->plane, p->domega,
-                                     p->eh, p->eh_time, b->stream),
+                                     p->time_tab, p->eh, p->eh_time, b->stream),
                 "omega-to-t kernel");
       p->time_valid = true;
       if (!e.done) BPM_BCUDA(b, cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming), "event");

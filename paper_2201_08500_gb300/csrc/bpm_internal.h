@@ -151,7 +151,7 @@ bool device_ready(int* sm_count);
 // outside stream capture, before the first launch on the current device.
 cudaError_t march_set_attributes();
 cudaError_t batch_set_attributes();
-cudaError_t setup_set_attributes();
+cudaError_t time_set_attributes();
 
 // Launchers (bpm_march.cu).  Return cudaSuccess or the launch error.
 int march_threads_per_channel(int n);
@@ -221,9 +221,25 @@ cudaError_t launch_tables(const SetupArgs& sa, const double* omega, const double
                           cudaStream_t s);
 cudaError_t launch_incident(const SetupArgs& sa, const double* omega, const double2* weight,
                             float2* e0, float2* eh, double* inc_norm, cudaStream_t s);
+
+// Frequency-to-time assembly (bpm_time.cu).  Shape of the transform over n
+// channels: len = n with radices up to 8, or (chirp) the power-of-two length of
+// Bluestein's form.
+struct TimeShape {
+  int n, len, chirp, n_pass;
+  unsigned char radix[16];
+};
+// False if n takes the direct sum (which needs no tables).
+bool time_shape(int n, TimeShape* s);
+// Elements of the tables of an n-channel transform (0: none), and their setup;
+// the plan keeps them, so that no run makes them again.
+size_t time_table_elems(int n);
+cudaError_t launch_time_tables(int n, double2* tt, cudaStream_t s);
 // Time response of channels first .. first + n_local - 1 of n_total ([n_total]
-// rows of plane values; the other channels count as zero).
+// rows of plane values; the other channels count as zero).  tt: the tables of
+// n_total (null: the direct sum).
 cudaError_t launch_omega_to_t(int n_total, int first, int n_local, long long plane,
-                              double domega, const float2* eh, double2* out, cudaStream_t s);
+                              double domega, const double2* tt, const float2* eh, double2* out,
+                              cudaStream_t s);
 
 }  // namespace bpm

@@ -1,5 +1,5 @@
 // Per-plan setup kernels of the BPM (FP64 arithmetic, run once per crystal /
-// pulse) and the frequency-to-time assembly.
+// pulse).  The frequency-to-time assembly is in bpm_time.cu.
 //
 //  deformation_kernel : c(x, z) = Pi(x, z) exp(+i h u(x, z))         (Eq. Authier);
 //                       Pi from the crystal's boundaries or a caller's mask
@@ -7,8 +7,6 @@
 //                       (Eqs. fov4, fov11, fov12, Zassenhaus-like factor)
 //  incident_kernel    : A+ = S g(x, y) exp(i (k sin theta_i - h/2) x), A- = 0
 //                       (beam of Section 3.1, spectral amplitude of Eq. ref:tdp)
-//  omega_to_t kernels : psi_h(t_j) = d_omega sum_i A-(omega_i) exp(-2 pi i (i - n/2) j / n)
-//                       (frequency reassembly after Eq. ref:tdp), FP64 accumulation
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -298,97 +296,7 @@ __global__ void incident_kernel(SetupArgs sa, const double* __restrict__ omega,
   }
 }
 
-// Frequency-to-time, n a power of two: per block COLS columns of the
-// [n][plane] spectrum, FP64 radix-2 transform in shared memory (bit-reversed
-// load, log2 n butterfly passes), output scaled by d_omega exp(2 pi i (n/2) j / n).
-// The plan holds channels first .. first + n_local - 1 of the n (a channel
-// shard, or all of them); the others enter as zeros, so the output is this
-// shard's part of the sum.
-// The n/2 twiddles W^m = exp(-2 pi i m / n) are computed once per block into
-// shared memory; stage len uses W^(kk n / len) (the same double as
-// exp(-2 pi i kk / len): both arguments are exact binary fractions).
-constexpr int kCols = 8;
-__global__ void omega_to_t_fft_kernel(int n, int logn, int first, int n_local, long long plane,
-                                      double domega, const float2* __restrict__ eh, double2* out) {
-  extern __shared__ double2 sm[];  // [n][kCols], then the twiddles [n/2]
-  double2* tw = sm + size_t(n) * kCols;
-  const long long x0 = (long long)blockIdx.x * kCols;
-  const int cols = int(min((long long)kCols, plane - x0));
-  for (int m = threadIdx.x; m < n / 2; m += blockDim.x) {
-    double s, co;
-    sincospi(-2.0 * double(m) / double(n), &s, &co);
-    tw[m] = make_double2(co, s);
-  }
-  for (int idx = threadIdx.x; idx < n * kCols; idx += blockDim.x) {
-    const int i = idx / kCols, c = idx % kCols;
-    const int ri = logn ? int(__brev(unsigned(i)) >> (32 - logn)) : 0;
-    double2 v = make_double2(0.0, 0.0);
-    const int li = i - first;
-    if (c < cols && li >= 0 && li < n_local) {
-      const float2 f = eh[(long long)li * plane + x0 + c];
-      v = make_double2(double(f.x), double(f.y));
-    }
-    sm[ri * kCols + c] = v;
-  }
-  __syncthreads();
-  for (int half = 1; half < n; half <<= 1) {
-    const int len = half * 2;
-    const int step = n / len;
-    for (int idx = threadIdx.x; idx < (n / 2) * kCols; idx += blockDim.x) {
-      const int bf = idx / kCols, c = idx % kCols;
-      const int grp = bf / half, kk = bf % half;
-      const int ia = grp * len + kk, ib = ia + half;
-      const double2 w = tw[kk * step];
-      const double2 u = sm[ia * kCols + c], v = sm[ib * kCols + c];
-      const double2 wv = make_double2(v.x * w.x - v.y * w.y, v.x * w.y + v.y * w.x);
-      sm[ia * kCols + c] = make_double2(u.x + wv.x, u.y + wv.y);
-      sm[ib * kCols + c] = make_double2(u.x - wv.x, u.y - wv.y);
-    }
-    __syncthreads();
-  }
-  const int ic = n / 2;
-  for (int idx = threadIdx.x; idx < n * kCols; idx += blockDim.x) {
-    const int j = idx / kCols, c = idx % kCols;
-    if (c >= cols) continue;
-    // exp(+2 pi i e / n) = conj(W^e), W^(e + n/2) = -W^e
-    const int e = int(((long long)ic * j) % n);
-    const double2 w0 = tw[e % ic];
-    const double sg = e < ic ? 1.0 : -1.0;
-    const double co = sg * w0.x, s = -sg * w0.y;
-    const double2 v = sm[j * kCols + c];
-    out[(long long)j * plane + x0 + c] =
-        make_double2(domega * (v.x * co - v.y * s), domega * (v.x * s + v.y * co));
-  }
-}
-
-// Direct FP64 sum for any n (used when n is not a power of two), over this
-// plan's channels first .. first + n_local - 1 of the n.
-__global__ void omega_to_t_direct_kernel(int n, int first, int n_local, long long plane,
-                                         double domega, const float2* __restrict__ eh,
-                                         double2* out) {
-  const long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (x >= plane) return;
-  const int ic = n / 2;
-  double re = 0.0, im = 0.0;
-  for (int li = 0; li < n_local; ++li) {
-    const int i = first + li;
-    const long long e = (((long long)(i - ic) * j) % n + n) % n;
-    double s, co;
-    sincospi(-2.0 * double(e) / double(n), &s, &co);
-    const float2 f = eh[(long long)li * plane + x];
-    re += double(f.x) * co - double(f.y) * s;
-    im += double(f.x) * s + double(f.y) * co;
-  }
-  out[(long long)j * plane + x] = make_double2(domega * re, domega * im);
-}
-
 }  // namespace
-
-cudaError_t setup_set_attributes() {
-  return cudaFuncSetAttribute(omega_to_t_fft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              200 * 1024);
-}
 
 cudaError_t launch_deformation(const SetupArgs& sa, const double* u_dev, float2* cfield,
                                cudaStream_t s) {
@@ -423,25 +331,6 @@ cudaError_t launch_tables3d(const SetupArgs& sa, const double* omega, const doub
 cudaError_t launch_incident(const SetupArgs& sa, const double* omega, const double2* weight,
                             float2* e0, float2* eh, double* inc_norm, cudaStream_t s) {
   incident_kernel<<<sa.n_ch, 256, 0, s>>>(sa, omega, weight, e0, eh, inc_norm);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_omega_to_t(int n_total, int first, int n_local, long long plane,
-                              double domega, const float2* eh, double2* out, cudaStream_t s) {
-  if (first < 0 || n_local < 0 || first + n_local > n_total) return cudaErrorInvalidValue;
-  const int n = n_total;
-  const bool pow2 = n > 0 && (n & (n - 1)) == 0;
-  const size_t smem = size_t(n) * kCols * sizeof(double2) + size_t(n / 2) * sizeof(double2);
-  if (pow2 && n >= 2 && smem <= 200 * 1024) {
-    int logn = 0;
-    while ((1 << logn) < n) ++logn;
-    const long long blocks = (plane + kCols - 1) / kCols;
-    omega_to_t_fft_kernel<<<int(blocks), 256, smem, s>>>(n, logn, first, n_local, plane, domega,
-                                                        eh, out);
-    return cudaGetLastError();
-  }
-  dim3 grid(unsigned((plane + 127) / 128), unsigned(n));
-  omega_to_t_direct_kernel<<<grid, 128, 0, s>>>(n, first, n_local, plane, domega, eh, out);
   return cudaGetLastError();
 }
 
