@@ -1530,7 +1530,14 @@ BPM_API bpm_status bpm_batch_run_graph(bpm_batch b) {
   BPM_NVTX();
   if (!b) return bfail(nullptr, BPM_ERR_INVALID_ARG, "null batch");
   uint64_t key = 1469598103934665603ull;
-  for (const auto& e : b->entries) key = (key ^ reinterpret_cast<uintptr_t>(e.plan)) * 1099511628211ull;
+  auto mix = [&key](uint64_t v) { key = (key ^ v) * 1099511628211ull; };
+  for (const auto& e : b->entries) {
+    mix(reinterpret_cast<uintptr_t>(e.plan));
+    // a shard declared since the capture has other time-response buffers
+    mix(reinterpret_cast<uintptr_t>(e.plan->eh_time));
+    mix(reinterpret_cast<uintptr_t>(e.plan->time_tab));
+    mix(uint64_t(e.plan->shard_first) << 32 | uint32_t(time_rows(e.plan)));
+  }
   if (!b->graph || key != b->graph_key) {
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;

@@ -54,6 +54,32 @@ __device__ __forceinline__ dc dsqrt(dc z) {
 
 __device__ __forceinline__ float2 to_f2(dc z) { return make_float2(float(z.re), float(z.im)); }
 
+// Nearest float (ties to even) of a double whose magnitude is a normal float
+// below 2^127, or zero, in integer instructions: the conversion instructions
+// between 64 and 32 bits run at the FP64 rate, which the tables are bound by.
+__device__ __forceinline__ float round_f32(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long a = b & 0x7FFFFFFFFFFFFFFFull;
+  const unsigned m = unsigned((a + 0x0FFFFFFFull + ((a >> 29) & 1)) >> 29) - (896u << 23);
+  return __uint_as_float((a ? m : 0u) | (unsigned(b >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ double widen_f64(float f) {
+  const unsigned b = __float_as_uint(f);
+  const unsigned long long a = ((unsigned long long)(b & 0x7FFFFFFFu) + (896ull << 23)) << 29;
+  return __longlong_as_double((long long)(a | ((unsigned long long)(b & 0x80000000u) << 32)));
+}
+// v as FP32 hi + lo, each rounded to nearest.
+__device__ __forceinline__ void split_f32(double v, float* hi, float* lo) {
+  const unsigned e = (unsigned(__double_as_longlong(v) >> 52)) & 0x7FFu;
+  if (e - (1023u - 60u) < 100u) {  // 2^-60 <= |v| < 2^40: lo is zero or a normal float too
+    *hi = round_f32(v);
+    *lo = round_f32(v - widen_f64(*hi));
+  } else {
+    *hi = float(v);
+    *lo = float(v - double(*hi));
+  }
+}
+
 // Spatial frequency of DFT bin m on an n-point grid of spacing d (Nyquist negative).
 __device__ __forceinline__ double qbin(int m, int n, double d) {
   const int mm = (m < n / 2) ? m : m - n;
@@ -142,14 +168,22 @@ __global__ void crystal_span_kernel(const float2* __restrict__ cfield, int nx, l
 }
 
 // Power series of J0(w) and G1(w) = 2 J1(w)/w in terms of w^2 (A&S 9.1.10).
+// It ends where neither a term nor any later one (each at most half the one
+// before, once |z| <= k^2 / 2) can change a sum: after a few terms of the w of
+// thin slices, instead of a serial chain of 39 that took 80 us.
 __device__ void bessel_j0_g1(dc w2, dc* j0, dc* g1) {
   const dc z = dscale(w2, -0.25);
+  const double az = fabs(z.re) + fabs(z.im);
   dc t0 = dmk(1, 0), t1 = dmk(1, 0), s0 = dmk(1, 0), s1 = dmk(1, 0);
   for (int k = 1; k < 40; ++k) {
     t0 = ddiv_real(dmul(t0, z), double(k) * k);
     t1 = ddiv_real(dmul(t1, z), double(k) * (k + 1));
     s0 = dadd(s0, t0);
     s1 = dadd(s1, t1);
+    const double tiny = (fabs(t0.re) + fabs(t0.im)) * 0x1p+54;
+    if (2.0 * az <= double(k) * k && tiny <= fabs(s0.re) && tiny <= fabs(s1.re) &&
+        (z.im == 0.0 || (tiny <= fabs(s0.im) && tiny <= fabs(s1.im))))
+      break;
   }
   *j0 = s0;
   *g1 = s1;
@@ -180,47 +214,103 @@ __device__ ChannelCoef channel_coef(const SetupArgs& sa, double kdz, double cos_
   return c;
 }
 
-// One block per channel.  Tables are written in the march kernel's order:
-// [ch][env][k][t] for the spectrum position p = 16 t + k, env 0 = E0 (+h/2), 1 = Eh (-h/2).
-__global__ void tables_kernel(SetupArgs sa, const double* __restrict__ omega,
-                              const double* __restrict__ gain, const int* __restrict__ rev,
-                              float4* tables, ChannelCoef* coef, int* bad) {
-  const int ch = blockIdx.x;
-  const int n = sa.nx;
-  const int T = n / 16;
-  const double k = omega[ch] / kC;
-  const double half_h = 0.5 * sa.h;
-  const double s_ratio = half_h / k;
+constexpr int kTabThreads = 128;
+constexpr int kTabMaxCh = 8;  // channels per block of tables_kernel
+
+// Coupling coefficients of channel / set `i` (set fastest), fractions cfr of dz.
+__device__ void store_coef(const SetupArgs& sa, const double* omega, int i, int n_sets,
+                           const double (&cfr)[2], ChannelCoef* coef, int* bad) {
+  const double k = omega[i / n_sets] / kC;
+  const double s_ratio = 0.5 * sa.h / k;
   if (!(s_ratio < 1.0)) {
-    if (threadIdx.x == 0) atomicExch(bad, 1);
+    if (bad) atomicExch(bad, 1);
     return;
   }
   const double cos_a = sqrt(1.0 - s_ratio * s_ratio);  // cos(alpha), Eq. fov3
-  const double kdz = k * sa.dz;
+  coef[i] = channel_coef(sa, k * sa.dz * cfr[i % n_sets], cos_a);
+}
+
+// Position of frequency bin f in the digit-reversed spectrum of n points: the
+// base-16 digits of f from the lowest, the last one of what remains.
+__device__ __forceinline__ int spectrum_position(int f, int n) {
+  int p = 0;
+  for (int l = n / 16; l >= 1; l /= 16) {
+    p += (f & 15) * l;
+    f >>= 4;
+    if (l < 16) {
+      if (l > 1) p += f;
+      break;
+    }
+  }
+  return p;
+}
+
+// Tables in the march kernel's order: [ch][env][k][t] for the spectrum position
+// p = 16 t + k, env 0 = E0 (+h/2), 1 = Eh (-h/2).  FP64 bound (two operations
+// a clock and SM), so:
+//  * the phase factor of (Eh, q) is that of (E0, -q) bit for bit, (q - h/2)^2 =
+//    (-q + h/2)^2, so one square root, division and sincos serve both; only the
+//    Nyquist bin, whose -q is not on the grid, has its own;
+//  * a thread keeps its bin for up to kTabMaxCh channels: q and the gains'
+//    reciprocals are divided out once;
+//  * a grid of 128-bin blocks also spreads a single channel over many SMs, and
+//    the coefficients (a serial chain) run in blocks of their own in front, one
+//    thread per channel.
+// 8192 bins x 512 channels: 1600 -> 771 us (about 100 FP64 instructions a pair
+// of entries); two sets of 4096 x 256: 660 -> 327 us; 48 plans of 512 x 1, one
+// after the other: 91 -> 20 us each.
+__global__ void __launch_bounds__(kTabThreads)
+    tables_kernel(SetupArgs sa, int coef_blocks, int cpb, const double* __restrict__ omega,
+                  const double* __restrict__ gain, const int* __restrict__ rev, float4* tables,
+                  ChannelCoef* coef, int* bad) {
   // fractions of dz of the propagations (tables) and couplings (coefficient
   // sets) of Eq. split-op: order 1: (1; 1); order 2: (1; 1/2); order 4:
   // (t, 1-2t; t/2, (1-t)/2) with t = 1/(2 - 2^(1/3))
-  const double t4 = 1.0 / (2.0 - cbrt(2.0));
+  const double t4 = sa.split_order == 4 ? 1.0 / (2.0 - cbrt(2.0)) : 0.0;
   const int n_sets = sa.split_order == 4 ? 2 : 1;
-  const double pf[2] = {sa.split_order == 4 ? t4 : 1.0, 1.0 - 2.0 * t4};
-  const double cfr[2] = {sa.split_order == 4 ? 0.5 * t4 : (sa.split_order == 2 ? 0.5 : 1.0),
-                         0.5 * (1.0 - t4)};
-  if (threadIdx.x < n_sets)
-    coef[size_t(ch) * n_sets + threadIdx.x] = channel_coef(sa, kdz * cfr[threadIdx.x], cos_a);
-  for (int set = 0; set < n_sets; ++set) {
-    float4* out = tables + (size_t(ch) * n_sets + set) * 2 * n;
-    for (int p = threadIdx.x; p < n; p += blockDim.x) {
-      const double q = qbin(rev[p], n, sa.dx);
-      const double scale = 1.0 / (double(n) * gain[p]);
-      const int t = p / 16, kk = p % 16;
-      for (int env = 0; env < 2; ++env) {
-        const double Q = env == 0 ? q + half_h : q - half_h;
-        dc P = tilted_propagator(k, Q * Q, sa.dz * pf[set]);
-        P = dscale(P, scale);
-        const float2 hi = to_f2(P);
-        const float2 lo = make_float2(float(P.re - double(hi.x)), float(P.im - double(hi.y)));
-        out[size_t(env) * n + size_t(kk) * T + t] = make_float4(hi.x, hi.y, lo.x, lo.y);
-      }
+  if (int(blockIdx.x) < coef_blocks) {
+    const double cfr[2] = {sa.split_order == 4 ? 0.5 * t4 : (sa.split_order == 2 ? 0.5 : 1.0),
+                           0.5 * (1.0 - t4)};
+    const int i = int(blockIdx.x) * 32 + threadIdx.x;
+    if (threadIdx.x < 32 && i < sa.n_ch * n_sets)
+      store_coef(sa, omega, i, n_sets, cfr, coef, bad);
+    return;
+  }
+  __shared__ double sk[kTabMaxCh];
+  const int n = sa.nx, T = n / 16, chunks = n / kTabThreads;
+  const int blk = int(blockIdx.x) - coef_blocks;
+  const int ch0 = (blk / chunks) * cpb, nch = min(cpb, sa.n_ch - ch0);
+  if (int(threadIdx.x) < nch) {
+    const double k = omega[ch0 + threadIdx.x] / kC;
+    sk[threadIdx.x] = 0.5 * sa.h / k < 1.0 ? k : -1.0;  // no Bragg solution: no tables
+  }
+  __syncthreads();
+  const int o = (blk % chunks) * kTabThreads + threadIdx.x;  // slot k T + t of env 0
+  const int p = 16 * (o % T) + o / T;
+  const int f = rev[p];
+  const int pm = spectrum_position((n - f) & (n - 1), n);    // where -q lives
+  const int om = (pm % 16) * T + pm / 16;
+  const double half_h = 0.5 * sa.h, q = qbin(f, n, sa.dx);
+  const double sc0 = 1.0 / (double(n) * gain[p]), sc1 = 1.0 / (double(n) * gain[pm]);
+  const double Q = q + half_h;
+  const bool nyquist = f == n / 2;
+  auto put = [](dc P, double scale, float4* dst) {
+    P = dscale(P, scale);
+    float4 v;
+    split_f32(P.re, &v.x, &v.z);
+    split_f32(P.im, &v.y, &v.w);
+    *dst = v;
+  };
+  for (int c = 0; c < nch; ++c) {
+    const double k = sk[c];
+    if (k < 0.0) continue;
+    for (int set = 0; set < n_sets; ++set) {
+      const double dz = sa.dz * (set ? 1.0 - 2.0 * t4 : sa.split_order == 4 ? t4 : 1.0);
+      float4* out = tables + (size_t(ch0 + c) * n_sets + set) * 2 * n;
+      dc P = tilted_propagator(k, Q * Q, dz);
+      put(P, sc0, out + o);
+      if (nyquist) P = tilted_propagator(k, (q - half_h) * (q - half_h), dz);
+      put(P, sc1, out + n + om);
     }
   }
 }
@@ -228,32 +318,35 @@ __global__ void tables_kernel(SetupArgs sa, const double* __restrict__ omega,
 // 3D: per channel and stored x-frequency column cs (px = 16 (cs % T) + cs / T),
 // the anchor exp(i dz (K - k)) / (nx ny g_x(px)), K = sqrt(k^2 - (qx +- h/2)^2),
 // as FP32 hi + lo, and the curvature factor -dz / (2 K) of the qy correction.
-__global__ void tables3d_kernel(SetupArgs sa, const double* __restrict__ omega,
-                                const double* __restrict__ gainx, const int* __restrict__ revx,
-                                float4* anchor, float* gcorr, ChannelCoef* coef) {
-  const int ch = blockIdx.x;
-  const int n = sa.nx;
-  const int T = n / 16;
+// Blocks of 128 columns of a channel; coefficients as in tables_kernel.
+__global__ void __launch_bounds__(kTabThreads)
+    tables3d_kernel(SetupArgs sa, int coef_blocks, const double* __restrict__ omega,
+                    const double* __restrict__ gainx, const int* __restrict__ revx, float4* anchor,
+                    float* gcorr, ChannelCoef* coef) {
+  if (int(blockIdx.x) < coef_blocks) {
+    const double cfr[2] = {sa.coupling_frac, 0.0};
+    const int i = int(blockIdx.x) * 32 + threadIdx.x;
+    if (threadIdx.x < 32 && i < sa.n_ch) store_coef(sa, omega, i, 1, cfr, coef, nullptr);
+    return;
+  }
+  const int n = sa.nx, T = n / 16, chunks = n / kTabThreads;
+  const int blk = int(blockIdx.x) - coef_blocks;
+  const int ch = blk / chunks, cs = (blk % chunks) * kTabThreads + threadIdx.x;
   const double k = omega[ch] / kC;
   const double half_h = 0.5 * sa.h;
-  const double s_ratio = half_h / k;
-  const double cos_a = sqrt(1.0 - s_ratio * s_ratio);
-  if (threadIdx.x == 0) coef[ch] = channel_coef(sa, k * sa.dz * sa.coupling_frac, cos_a);
-  for (int cs = threadIdx.x; cs < n; cs += blockDim.x) {
-    const int px = 16 * (cs % T) + cs / T;
-    const double qx = qbin(revx[px], n, sa.dx);
-    const double scale = 1.0 / (double(n) * double(sa.ny) * gainx[px]);
-    for (int env = 0; env < 2; ++env) {
-      const double Q = env == 0 ? qx + half_h : qx - half_h;
-      const double K2 = k * k - Q * Q;
-      dc P = tilted_propagator(k, Q * Q, sa.dz);
-      P = dscale(P, scale);
-      const float2 hi = to_f2(P);
-      const float2 lo = make_float2(float(P.re - double(hi.x)), float(P.im - double(hi.y)));
-      const size_t o = (size_t(ch) * 2 + env) * n + cs;
-      anchor[o] = make_float4(hi.x, hi.y, lo.x, lo.y);
-      gcorr[o] = K2 > 0.0 ? float(-sa.dz / (2.0 * sqrt(K2))) : 0.f;
-    }
+  const int px = 16 * (cs % T) + cs / T;
+  const double qx = qbin(revx[px], n, sa.dx);
+  const double scale = 1.0 / (double(n) * double(sa.ny) * gainx[px]);
+  for (int env = 0; env < 2; ++env) {
+    const double Q = env == 0 ? qx + half_h : qx - half_h;
+    const double K2 = k * k - Q * Q;
+    dc P = tilted_propagator(k, Q * Q, sa.dz);
+    P = dscale(P, scale);
+    const float2 hi = to_f2(P);
+    const float2 lo = make_float2(float(P.re - double(hi.x)), float(P.im - double(hi.y)));
+    const size_t o = (size_t(ch) * 2 + env) * n + cs;
+    anchor[o] = make_float4(hi.x, hi.y, lo.x, lo.y);
+    gcorr[o] = K2 > 0.0 ? float(-sa.dz / (2.0 * sqrt(K2))) : 0.f;
   }
 }
 
@@ -317,14 +410,23 @@ cudaError_t launch_crystal_span(const float2* cfield, int nx, long long rows, in
 cudaError_t launch_tables(const SetupArgs& sa, const double* omega, const double* gain,
                           const int* rev, float4* tables, ChannelCoef* coef, int* bad,
                           cudaStream_t s) {
-  tables_kernel<<<sa.n_ch, 256, 0, s>>>(sa, omega, gain, rev, tables, coef, bad);
+  const int sets = sa.split_order == 4 ? 2 : 1, coef_blocks = (sa.n_ch * sets + 31) / 32;
+  // as many channels a block as leave eight blocks an SM (16 warps keep FP64 busy)
+  const long long chunks = sa.nx / kTabThreads;
+  int cpb = kTabMaxCh;
+  while (cpb > 1 && chunks * ((sa.n_ch + cpb - 1) / cpb) < 152 * 8) cpb /= 2;
+  const long long blocks = coef_blocks + chunks * ((sa.n_ch + cpb - 1) / cpb);
+  tables_kernel<<<unsigned(blocks), kTabThreads, 0, s>>>(sa, coef_blocks, cpb, omega, gain, rev,
+                                                         tables, coef, bad);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tables3d(const SetupArgs& sa, const double* omega, const double* gainx,
                             const int* revx, float4* anchor, float* gcorr, ChannelCoef* coef,
                             cudaStream_t s) {
-  tables3d_kernel<<<sa.n_ch, 256, 0, s>>>(sa, omega, gainx, revx, anchor, gcorr, coef);
+  const int coef_blocks = (sa.n_ch + 31) / 32;
+  tables3d_kernel<<<coef_blocks + sa.n_ch * (sa.nx / kTabThreads), kTabThreads, 0, s>>>(
+      sa, coef_blocks, omega, gainx, revx, anchor, gcorr, coef);
   return cudaGetLastError();
 }
 
