@@ -257,6 +257,7 @@ struct bpm_plan_s {
   double2* eh_time = nullptr;
   double2* time_tab = nullptr;   // tables of the frequency-to-time transform (null: direct sum)
   int* dflag = nullptr;
+  NormScratch* norm_scratch = nullptr;
   double* u_tmp = nullptr;
   float* gcorr = nullptr;        // 3D: curvature factor per column
   float2* spec = nullptr;        // 3D: transposed x-spectra of both envelopes [2][ch][nx][ny]
@@ -316,7 +317,7 @@ void free_plan_buffers(bpm_plan p) {
                   p->rev,    p->gain,    p->omega, p->weight, p->inc_norm, p->refl,
                   p->trans,  p->eh_time, p->dflag, p->u_tmp,  p->gcorr,    p->twy,
                   p->qy,     p->spec,    p->twx3,  p->twiddle_t, p->twiddle_p, p->mask,
-                  p->cspan,  p->time_tab};
+                  p->cspan,  p->time_tab, p->norm_scratch};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->ev0) cudaEventDestroy(p->ev0);
@@ -391,7 +392,7 @@ size_t plan_bytes(const bpm_grid& g, int n_ch) {
   b += sets * n_ch * sizeof(ChannelCoef);
   b += size_t(g.nx) * (sizeof(float2) + sizeof(int) + sizeof(double));
   if (g.dims == 2) b += 3 * size_t(g.nx) * sizeof(float2);  // thread-order twiddles, pairs
-  b += size_t(n_ch) * (5 * sizeof(double) + sizeof(double2));
+  b += size_t(n_ch) * (5 * sizeof(double) + sizeof(double2)) + sizeof(NormScratch);
   b += (nf + time_table_elems(n_ch)) * sizeof(double2);  // time response, its transform's tables
   return b;
 }
@@ -413,7 +414,8 @@ cudaError_t enqueue_pulse(bpm_plan p) {
                       : launch_tables(p->sa, p->omega, p->gain, p->rev, p->tables, p->coef,
                                       p->dflag, p->stream);
   if (e != cudaSuccess) return e;
-  e = launch_incident(p->sa, p->omega, p->weight, p->e0, p->eh, p->inc_norm, p->stream);
+  e = launch_incident(p->sa, p->omega, p->weight, p->e0, p->eh, p->inc_norm,
+                      p->norm_scratch, p->stream);
   p->z = 0;
   p->time_valid = false;
   return e;
@@ -494,6 +496,7 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
   check(dalloc(&p->eh_time, nf), "alloc time response");
   check(dalloc(&p->time_tab, time_table_elems(n_channels)), "alloc time tables");
   check(dalloc(&p->dflag, size_t(4)), "alloc status");
+  check(dalloc(&p->norm_scratch, size_t(1)), "alloc norm parts");
   if (g.dims == 3) {
     check(dalloc(&p->gcorr, size_t(n_channels) * 2 * g.nx), "alloc curvature factors");
     check(dalloc(&p->spec, 2 * nf), "alloc spectrum buffers");
@@ -529,6 +532,7 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
                         p->stream),
         "upload gain");
   check(cudaMemsetAsync(p->dflag, 0, sizeof(int) * 4, p->stream), "clear status");
+  check(cudaMemsetAsync(p->norm_scratch, 0, sizeof(NormScratch), p->stream), "clear norm parts");
   check(launch_time_tables(n_channels, p->time_tab, p->stream), "time tables");
   std::vector<float2> qyt;
   if (g.dims == 3) {

@@ -219,8 +219,16 @@ cudaError_t launch_deformation(const SetupArgs& sa, const double* u_dev, float2*
 cudaError_t launch_tables(const SetupArgs& sa, const double* omega, const double* gain,
                           const int* rev, float4* tables, ChannelCoef* coef, int* bad,
                           cudaStream_t s);
+// Parts of the incident field's norm (one per 256 cells in 2D, per 64 x 64 in
+// 3D) and the count of blocks that have written theirs: zero before the first
+// launch, and again after each.
+struct NormScratch {
+  int arrived;
+  double part[256];
+};
 cudaError_t launch_incident(const SetupArgs& sa, const double* omega, const double2* weight,
-                            float2* e0, float2* eh, double* inc_norm, cudaStream_t s);
+                            float2* e0, float2* eh, double* inc_norm, NormScratch* scratch,
+                            cudaStream_t s);
 
 // Frequency-to-time assembly (bpm_time.cu).  Shape of the transform over n
 // channels: len = n with radices up to 8, or (chirp) the power-of-two length of

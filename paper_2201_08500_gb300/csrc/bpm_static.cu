@@ -45,7 +45,8 @@ constexpr size_t kOffWeight = kOffOmega + align256(sizeof(double) * kStaticMaxCh
 constexpr size_t kOffNorm = kOffWeight + align256(sizeof(double2) * kStaticMaxChannels);
 constexpr size_t kOffTrans = kOffNorm + align256(sizeof(double) * kStaticMaxChannels);
 constexpr size_t kOffFlag = kOffTrans + align256(sizeof(double) * kStaticMaxChannels);
-constexpr size_t kStaticBytes = kOffFlag + 256;
+constexpr size_t kOffNormParts = kOffFlag + 256;
+constexpr size_t kStaticBytes = kOffNormParts + align256(sizeof(NormScratch));
 
 __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
@@ -177,7 +178,7 @@ BPM_API bpm_status bpm_run_noalloc(const bpm_grid* grid, int n_channels,
   const int* h_rev;
   const double* h_gain;
   fft_host_constants(g.nx, &h_tw, &h_rev, &h_gain);
-  // every region below is rewritten in full by this call; only the flag must start at zero
+  // every region below is rewritten in full by this call; only the flag and the norm parts must start at zero
   BPM_SCUDA(cudaMemcpyAsync(twiddle, h_tw, sizeof(float2) * g.nx, cudaMemcpyHostToDevice, st),
             "upload twiddles");
   BPM_SCUDA(cudaMemcpyAsync(rev, h_rev, sizeof(int) * g.nx, cudaMemcpyHostToDevice, st),
@@ -190,13 +191,14 @@ BPM_API bpm_status bpm_run_noalloc(const bpm_grid* grid, int n_channels,
   BPM_SCUDA(cudaMemcpyAsync(d_weight, weight_re_im, sizeof(double2) * n_channels,
                             cudaMemcpyHostToDevice, st),
             "upload weights");
-  BPM_SCUDA(cudaMemsetAsync(flag, 0, sizeof(int), st), "clear flag");
+  BPM_SCUDA(cudaMemsetAsync(flag, 0, 256 + sizeof(NormScratch), st), "clear flag and norm parts");
 
   float2* e0 = static_cast<float2*>(e0_dev);
   float2* eh = static_cast<float2*>(eh_dev);
   BPM_SCUDA(launch_deformation(sa, u_field_dev, cfield, st), "deformation kernel");
   BPM_SCUDA(launch_tables(sa, d_omega, gain, rev, tables, coef, flag, st), "tables kernel");
-  BPM_SCUDA(launch_incident(sa, d_omega, d_weight, e0, eh, inc_norm, st), "incident kernel");
+  BPM_SCUDA(launch_incident(sa, d_omega, d_weight, e0, eh, inc_norm,
+                            reinterpret_cast<NormScratch*>(base + kOffNormParts), st), "incident kernel");
   MarchArgs a;
   a.tables = tables;
   a.coef = coef;

@@ -59,3 +59,37 @@ def test_channel_groups_of_the_setup(nx, n_ch):
         assert np.array_equal(q.e0()[0], e0[ch]) and np.array_equal(q.eh()[0], eh[ch])
         assert q.reflectivity()[0][0] == R[ch]
         q.close()
+
+
+@pytest.mark.parametrize("dims,nx,ny,n_ch,zx", [(2, 256, 1, 1, 0.0), (2, 512, 1, 9, 3e-4),
+                                                (2, 4096, 1, 309, 0.0), (2, 8192, 1, 3, -2e-4),
+                                                (3, 256, 512, 2, 0.0), (3, 1024, 256, 3, 4e-4)])
+def test_incident_field_and_norm(dims, nx, ny, n_ch, zx):
+    """Every cell of the incident field against the formula in FP64, from cells
+    that round to zero to amplitudes far from one, and the norm through T."""
+    w = workloads.large_3d(n_ch=n_ch, nx=nx, ny=ny, nz=1, with_u=False) if dims == 3 else \
+        deformed_small(nx, nz=1, n_ch=n_ch, seed=2)
+    w.zx, w.zR = zx, 1e-3
+    w.w0 = (6 if n_ch > 8 else nx // 20) * w.dx
+    rng = np.random.default_rng(nx)
+    w.S = rng.standard_normal(n_ch) * 10.0 ** rng.integers(-24, 4, n_ch) * np.exp(
+        1j * rng.uniform(0, 6, n_ch))
+    p = bpm.plan_from_workload(w)
+    p.run(0)
+    p.sync()
+    got, R, T = p.e0().reshape(n_ch, ny, nx), *p.reflectivity()[:2]
+    assert not p.eh().any()
+    p.close()
+    x = np.arange(nx) * w.dx
+    y = (np.arange(ny) - ny // 2) * w.dy if dims == 3 else np.zeros(1)
+    den = 1.0 + 1j * zx / w.zR
+    r2 = ((x - w.x0)[None, :] ** 2 + y[:, None] ** 2) / w.w0 ** 2
+    g = np.exp(-r2 / den) / (den if dims == 3 else np.sqrt(den))
+    h = 4.0 * np.pi * np.sin(w.theta_B) / w.lambda_B
+    dq = w.omega / workloads.C_LIGHT * np.sin(w.theta_i) - 0.5 * h
+    want = w.S[:, None, None] * g * np.exp(1j * dq[:, None, None] * x)
+    # dq is a difference of numbers 1e5 times larger: its FP64 rounding (8e-6 per
+    # metre) moves the phase by at most 1e-7 over the grid; FP32 rounds to 6e-8
+    # (1e-45 where it is denormal)
+    assert np.max(np.abs(got - want) - 3e-7 * np.abs(want)) <= 2e-45
+    assert np.all(R == 0.0) and np.max(np.abs(T - 1.0)) < 2e-7
