@@ -1331,12 +1331,17 @@ bpm_status enqueue_round(bpm_batch b, RoundSlot& r, int chunk) {
     steps[k] = std::min(chunk, p->grid.nz - p->z);
     const int G = batch_item_channels(n, p->grid.split_order);
     const int q = batch_queue(n, p->grid.split_order);
-    for (int c0 = 0; c0 < p->n_ch; c0 += G) {
+    for (int c0 = 0; c0 < p->n_ch;) {
+      const int left = std::min(G, p->n_ch - c0);
+      int qs = q;
+      const bool single = G > 1 && batch_singles(n, p->grid.split_order, left, &qs);
+      const int take = single ? 1 : left;
       Tmp t;
       t.it = BatchItem{k, c0, n, 0};
-      t.cost = double(steps[k]) * n * std::min(G, p->n_ch - c0) * std::log2(double(n));
-      t.q = q;
+      t.cost = double(steps[k]) * n * take * std::log2(double(n));
+      t.q = single ? qs : q;
       tmp.push_back(t);
+      c0 += take;
     }
   }
   // launch rank of each queue: the longest items (Nx = 8192, every order) first,
@@ -1344,7 +1349,9 @@ bpm_status enqueue_round(bpm_batch b, RoundSlot& r, int chunk) {
   static constexpr int kOrder[kQueueCount] = {
       kQueueTm8192,   kQueueTm8192s2, kQueueBig4,     kQueueTm4096,   kQueueTm4096s2,
       kQueuePk4096s4, kQueueTm2048,   kQueueTm2048s2, kQueuePk2048s4, kQueueTm1024,
-      kQueuePk1024s4, kQueueSmall,    kQueueSmall2,   kQueueSmall4};
+      kQueuePk1024s4, kQueueQuad1024s2, kQueueSmall,  kQueueSmall2,   kQueueSmall4,
+      kQueueQuad512,  kQueueQuad512s2, kQueueQuad512s4, kQueueQuad256, kQueueQuad256s2,
+      kQueueQuad256s4};
   int rank[kQueueCount];
   for (int i = 0; i < kQueueCount; ++i) rank[kOrder[i]] = i;
   std::stable_sort(tmp.begin(), tmp.end(), [&rank](const Tmp& x, const Tmp& y) {
@@ -1549,8 +1556,7 @@ BPM_API bpm_status bpm_batch_run_graph(bpm_batch b) {
     // allocations happen before the capture: staging for every item, completion events
     int n_items = 0;
     for (auto& e : b->entries) {
-      const int G = batch_item_channels(e.plan->grid.nx, e.plan->grid.split_order);
-      n_items += (e.plan->n_ch + G - 1) / G;
+      n_items += e.plan->n_ch;  // at most: an item has one channel or more
       if (!e.done) BPM_BCUDA(b, cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming), "event");
     }
     BPM_BCUDA(b, slot_reserve(b->graph_slot, int(b->entries.size()), n_items), "graph staging");

@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "bpm_parked.cuh"
+#include "bpm_quad.cuh"
 #include "bpm_resident.cuh"
 
 namespace bpm {
@@ -174,7 +175,44 @@ __global__ void __launch_bounds__(N / 16, 512 / (N / 16))
   }
 }
 
+// Single channels at Nx <= 1024 with 8 Nx/16 threads each (bpm_quad.cuh).
+template <int N, int SPLIT>
+__global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>::kThreads)
+    batch_kernel_quad(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
+                      int n_items, int* counter) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int s_item;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
+    __syncthreads();
+    const int it = s_item;
+    if (it >= n_items) break;
+    const BatchItem item = items[it];
+    Quad<N, SPLIT>::march_channel(plans[item.plan], item.ch0, smem);
+  }
+}
+
 }  // namespace
+
+// A resident item takes the time of a full one however few channels it has
+// (us a step: 256 points 2.9, 512 points 4.7; Strang 4.4, 5.8, 1024 points
+// 5.65; fourth order 10.3, 15.6), a single channel of the other form 0.25,
+// 0.65; 0.275, 0.70, 1.97; 0.85, 2.29 of an SM's time.
+bool batch_singles(int n, int split_order, int left, int* queue) {
+  int most = 0;
+  if (split_order == 1) {
+    most = n == 256 ? 11 : n == 512 ? 7 : 0;
+    *queue = n == 256 ? kQueueQuad256 : kQueueQuad512;
+  } else if (split_order == 2) {
+    most = n == 256 ? 15 : n == 512 ? 8 : n == 1024 ? 2 : 0;
+    *queue = n == 256 ? kQueueQuad256s2 : n == 512 ? kQueueQuad512s2 : kQueueQuad1024s2;
+  } else {
+    most = n == 256 ? 12 : n == 512 ? 6 : 0;
+    *queue = n == 256 ? kQueueQuad256s4 : kQueueQuad512s4;
+  }
+  return left <= most;
+}
 
 int batch_group(int n) { return n == 8192 ? 1 : kSmallThreads / (n / 16); }
 
@@ -215,6 +253,12 @@ int batch_blocks_per_sm(int queue) {
     case kQueuePk2048s4:
     case kQueueTm1024: return 4;
     case kQueuePk1024s4: return 8;
+    case kQueueQuad256:
+    case kQueueQuad256s2:
+    case kQueueQuad256s4: return 6;
+    case kQueueQuad512:
+    case kQueueQuad512s2:
+    case kQueueQuad512s4: return 3;
     default: return 1;
   }
 }
@@ -232,6 +276,13 @@ template <int N, int SPLIT>
 void pk_launch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
                int blocks, cudaStream_t s) {
   batch_kernel_pk<N, SPLIT><<<blocks, N / 16, Parked<N, SPLIT>::smem_bytes(), s>>>(
+      plans, items, n_items, counter);
+}
+
+template <int N, int SPLIT>
+void quad_launch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
+                 int blocks, cudaStream_t s) {
+  batch_kernel_quad<N, SPLIT><<<blocks, Quad<N, SPLIT>::kThreads, Quad<N, SPLIT>::smem_bytes(), s>>>(
       plans, items, n_items, counter);
 }
 
@@ -279,6 +330,13 @@ cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_i
     case kQueueBig4:
       batch_kernel_8192<4><<<blocks, 512, big_smem, s>>>(plans, items, n_items, counter);
       break;
+    case kQueueQuad256: quad_launch<256, 1>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueQuad512: quad_launch<512, 1>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueQuad256s2: quad_launch<256, 2>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueQuad512s2: quad_launch<512, 2>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueQuad1024s2: quad_launch<1024, 2>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueQuad256s4: quad_launch<256, 4>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueQuad512s4: quad_launch<512, 4>(plans, items, n_items, counter, blocks, s); break;
     default:
       return cudaErrorInvalidValue;
   }

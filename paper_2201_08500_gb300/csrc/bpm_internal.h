@@ -132,11 +132,18 @@ enum BatchQueue {
   kQueuePk1024s4,    // fourth order, Nx = 1024: parked form, L2 tables, 8 blocks / SM
   kQueueTm1024,      // first order, Nx = 1024: parked form, TMEM tables, two channels a
                      // block, 4 blocks / SM
+  // single channels at Nx <= 512 (Strang: 1024): 8 Nx/16 threads a channel (bpm_quad.cuh)
+  kQueueQuad256, kQueueQuad512,
+  kQueueQuad256s2, kQueueQuad512s2, kQueueQuad1024s2,
+  kQueueQuad256s4, kQueueQuad512s4,
   kQueueCount
 };
 int batch_group(int n);                               // channels per block of the resident kernels
 int batch_item_channels(int n, int split_order);      // channels per item
 int batch_queue(int n, int split_order);
+// Items of a plan's last `left` channels (fewer than an item's channels, or a
+// full item): singles in queue *queue (true) or one resident item.
+bool batch_singles(int n, int split_order, int left, int* queue);
 int batch_blocks_per_sm(int queue);
 cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
                          int queue, int blocks, cudaStream_t s);
@@ -159,6 +166,10 @@ int march_max_group(int n);
 size_t march_smem_bytes(int n, int group);
 cudaError_t launch_march(int n, int group, int blocks, const MarchArgs& a, cudaStream_t s);
 cudaError_t launch_march_strang(int n, int group, int blocks, const MarchArgs& a, cudaStream_t s);
+// The march with 8 n/16 threads a channel (bpm_march_quad.cu), n <= 1024, every
+// order: launch_march takes it for one channel a block where it is the faster.
+bool march_quad_use(int n, int split_order, int n_ch, int sms);
+cudaError_t launch_march_quad(int n, const MarchArgs& a, cudaStream_t s);
 // Second form of the first-order march: propagator tables and stage twiddles
 // read from L2 instead of shared memory / registers, at most 128 registers, so
 // that two blocks (two channel groups at independent FFT phases) share an SM.

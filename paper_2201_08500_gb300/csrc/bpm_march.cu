@@ -63,6 +63,9 @@ cudaError_t march_set_attributes() {
 }
 
 cudaError_t launch_march(int n, int group, int blocks, const MarchArgs& a, cudaStream_t s) {
+  int sms = 0;
+  if (group == 1 && device_ready(&sms) && march_quad_use(n, a.split_order, a.n_ch, sms))
+    return launch_march_quad(n, a, s);
   if (a.split_order == 2) return launch_march_strang(n, group, blocks, a, s);
   if (a.split_order == 4) return launch_march_split4(n, group, blocks, a, s);
 #define BPM_LAUNCH_CASE(NN, GG) \

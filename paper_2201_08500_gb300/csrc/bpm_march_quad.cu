@@ -1,0 +1,55 @@
+// Launches of the march with 8 N/16 threads a channel (bpm_quad.cuh).
+#include <cuda_runtime.h>
+
+#include "bpm_quad.cuh"
+
+namespace bpm {
+
+namespace {
+
+template <int N, int SPLIT>
+__global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>::kThreads)
+    march_quad_kernel(MarchArgs A) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  Quad<N, SPLIT>::run(A, smem);
+}
+
+template <int N, int SPLIT>
+cudaError_t launch_one(const MarchArgs& a, cudaStream_t s) {
+  march_quad_kernel<N, SPLIT>
+      <<<a.n_ch, Quad<N, SPLIT>::kThreads, Quad<N, SPLIT>::smem_bytes(), s>>>(a);
+  return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t launch_order(const MarchArgs& a, cudaStream_t s) {
+  if (a.split_order == 2) return launch_one<N, 2>(a, s);
+  if (a.split_order == 4) return launch_one<N, 4>(a, s);
+  return launch_one<N, 1>(a, s);
+}
+
+}  // namespace
+
+// The step times of the forms for n_ch channels, in us (measured over 1 ... 2500
+// channels, 152 SMs).  Up to 3 (256, 512 points) or 1 (1024) channels an SM
+// this form ends in 0.7, 1.0 and 1.8 us; beyond, it takes its share of an SM's
+// time per channel, and the resident form a whole wave of 16, 8 or 4 channels
+// an SM whether full or not.  E.g. first order, 512 points: 201 channels 1.45
+// against 3.85, 760 3.7 against 4.05, 1024 4.5 against 4.2.
+bool march_quad_use(int n, int split_order, int n_ch, int sms) {
+  const int o = split_order == 1 ? 0 : split_order == 2 ? 1 : 2;
+  static constexpr double each[3][3] = {{0.25, 0.275, 0.85}, {0.65, 0.70, 2.29}, {1.79, 1.97, 5.4}};
+  static constexpr double wave[3][3] = {{2.9, 4.35, 10.3}, {4.2, 5.2, 14.3}, {4.2, 5.2, 14.4}};
+  if (n > 1024 || n_ch < 1 || sms < 1) return false;
+  const int i = n == 256 ? 0 : n == 512 ? 1 : 2, per = n == 256 ? 16 : n == 512 ? 8 : 4;
+  return each[i][o] * ((n_ch + sms - 1) / sms) < wave[i][o] * ((n_ch + per * sms - 1) / (per * sms));
+}
+
+cudaError_t launch_march_quad(int n, const MarchArgs& a, cudaStream_t s) {
+  if (n == 256) return launch_order<256>(a, s);
+  if (n == 512) return launch_order<512>(a, s);
+  if (n == 1024) return launch_order<1024>(a, s);
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace bpm

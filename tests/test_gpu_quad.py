@@ -1,0 +1,62 @@
+"""The march with 8 Nx/16 threads a channel (few channels) against the grouped resident form."""
+import numpy as np
+import pytest
+
+from paper_2201_08500_gb300 import bpm
+from test_gpu_parity import deformed_small
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("order", [1, 2, 4])
+@pytest.mark.parametrize("nx,n_ch,maxg", [(256, 1, 16), (256, 35, 16), (512, 1, 8), (512, 160, 8),
+                                          (1024, 1, 4), (1024, 155, 4)])
+def test_few_channels_give_the_resident_forms_bits(nx, n_ch, maxg, order):
+    """Fields and reflectivities bitwise equal; a split run ends where a whole one does."""
+    w = deformed_small(nx, nz=61, n_ch=n_ch, seed=nx + order)
+    w.split_order = order
+    out = []
+    for group, steps in ((maxg, (61,)), (1, (61,)), (1, (1, 40, 20))):
+        p = bpm.plan_from_workload(w)
+        p.set_launch(form=0, channels_per_block=group)
+        for n in steps:
+            p.run(n)
+        p.sync()
+        out.append((p.e0(), p.eh(), *p.reflectivity()[:2]))
+        p.close()
+    for got in out[1:]:
+        for a, b in zip(out[0], got):
+            assert np.array_equal(a, b)
+
+
+def test_work_queue_singles_and_full_items_give_the_plans_bits():
+    """Plans of small grids in one batch: full resident items and the remainders
+    on either side of the line to single channels, each as marched alone."""
+    ws = []
+    for nx, order, counts in ((256, 1, (1, 27, 28)), (256, 2, (31,)), (256, 4, (12, 13)),
+                              (512, 1, (1, 15, 16)), (512, 2, (9,)), (512, 4, (6, 15)),
+                              (1024, 2, (2, 7))):
+        for n_ch in counts:
+            w = deformed_small(nx, nz=20 + n_ch, n_ch=n_ch, seed=n_ch)
+            w.split_order = order
+            ws.append(w)
+    want = []
+    for w in ws:
+        p = bpm.plan_from_workload(w)
+        p.run()
+        p.sync()
+        want.append((p.e0(), p.eh(), p.reflectivity()[0]))
+        p.close()
+    b = bpm.Batch()
+    plans = [bpm.plan_from_workload(w) for w in ws]
+    for p in plans:
+        b.submit(p)
+    b.step(13)
+    b.run()
+    b.sync()
+    for p, (e0, eh, R) in zip(plans, want):
+        assert np.array_equal(p.e0(), e0) and np.array_equal(p.eh(), eh)
+        assert np.array_equal(p.reflectivity()[0], R)
+    b.close()
+    for p in plans:
+        p.close()
