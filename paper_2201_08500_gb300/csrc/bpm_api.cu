@@ -239,6 +239,7 @@ struct bpm_plan_s {
 
   // device buffers
   float2* cfield = nullptr;
+  int* ext = nullptr;     // 2D: crystal extent of all rows (MarchArgs::ext)
   int2* cspan = nullptr;  // 3D: [nz][ny] crystal extent of each deformation row
   float2* e0 = nullptr;
   float2* eh = nullptr;
@@ -317,7 +318,7 @@ void free_plan_buffers(bpm_plan p) {
                   p->rev,    p->gain,    p->omega, p->weight, p->inc_norm, p->refl,
                   p->trans,  p->eh_time, p->dflag, p->u_tmp,  p->gcorr,    p->twy,
                   p->qy,     p->spec,    p->twx3,  p->twiddle_t, p->twiddle_p, p->mask,
-                  p->cspan,  p->time_tab, p->norm_scratch};
+                  p->cspan,  p->time_tab, p->norm_scratch, p->ext};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->ev0) cudaEventDestroy(p->ev0);
@@ -399,11 +400,7 @@ size_t plan_bytes(const bpm_grid& g, int n_ch) {
 
 // Re-derive the deformation factor of the plan from its stored displacement.
 cudaError_t enqueue_crystal(bpm_plan p) {
-  cudaError_t e = launch_deformation(p->sa, p->u_dev, p->cfield, p->stream);
-  if (e != cudaSuccess || p->grid.dims != 3) return e;
-  // 3D: the row pass loads each deformation row only inside its crystal extent
-  return launch_crystal_span(p->cfield, p->grid.nx, (long long)p->grid.nz * p->grid.ny, p->cspan,
-                             p->stream);
+  return launch_deformation(p->sa, p->u_dev, p->cfield, p->cspan, p->ext, p->stream);
 }
 
 // Tables, coefficients and incident field from the stored pulse; march back to z = 0.
@@ -478,6 +475,7 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
   };
   check(dalloc(&p->cfield, size_t(g.nz) * p->plane), "alloc deformation field");
   if (g.dims == 3) check(dalloc(&p->cspan, size_t(g.nz) * g.ny), "alloc crystal extents");
+  if (g.dims == 2) check(dalloc(&p->ext, size_t(2)), "alloc crystal extent");
   check(dalloc(&p->e0, nf), "alloc E0");
   check(dalloc(&p->eh, nf), "alloc Eh");
   const size_t sets = g.split_order == 4 ? 2 : 1;  // Eq. split-op order 4: two of each
@@ -793,6 +791,7 @@ BPM_API bpm_status bpm_run(bpm_plan p, int n_steps) {
   a.twiddle_t = p->twiddle_t;
   a.twiddle_p = p->twiddle_p;
   a.cfield = p->cfield;
+  a.ext = p->ext;
   a.e0 = p->e0;
   a.eh = p->eh;
   a.inc_norm = p->inc_norm;
@@ -1295,6 +1294,7 @@ MarchArgs march_args(bpm_plan p, int n_steps) {
   a.twiddle_t = p->twiddle_t;
   a.twiddle_p = p->twiddle_p;
   a.cfield = p->cfield;
+  a.ext = p->ext;
   a.e0 = p->e0;
   a.eh = p->eh;
   a.inc_norm = p->inc_norm;

@@ -60,6 +60,7 @@ struct MarchArgs {
   const float2* twiddle_t;   // stage twiddles in thread order (kernels that read them from memory)
   const float2* twiddle_p;   // the same in thread-ordered pairs (parked forms, 128-bit loads)
   const float2* cfield;      // [nz][N] Pi(x, z) exp(+i h u(x, z)); 0 outside the crystal
+  const int* ext;            // {lo, -hi} of the crystal's x over all rows (launch_deformation)
   float2* e0;                // [n_ch][N]
   float2* eh;                // [n_ch][N]
   const double* inc_norm;    // [n_ch] sum |A+(z=0)|^2
@@ -218,15 +219,13 @@ cudaError_t launch_reduce3d(const float2* e0, const float2* eh, long long plane,
 cudaError_t launch_tables3d(const SetupArgs& sa, const double* omega, const double* gainx,
                             const int* revx, float4* anchor, float* gcorr, ChannelCoef* coef,
                             cudaStream_t s);
-// Extent of the crystal in each of `rows` deformation rows of nx cells:
-// span[r] = {first x with c != 0, last such x + 1}, {0, 0} for a row without
-// crystal.  The 3D row pass loads a row's c only inside it (c = 0 outside).
-// (The 1D marches load their rows unconditionally: guarding those loads by
-// the extent measured slower there.)
-cudaError_t launch_crystal_span(const float2* cfield, int nx, long long rows, int2* span,
-                                cudaStream_t s);
+// Deformation factor; span (3D, or null): {first x with c != 0, last such x + 1}
+// of each [nz][ny] row, {0, 0} for a row without crystal; ext (2D, or null):
+// their union as {lo, -hi}, or kExtNone twice for no crystal at all.
+constexpr int kExtNoneByte = 0x7F;
+constexpr int kExtNone = 0x7F7F7F7F;
 cudaError_t launch_deformation(const SetupArgs& sa, const double* u_dev, float2* cfield,
-                               cudaStream_t s);
+                               int2* span, int* ext, cudaStream_t s);
 cudaError_t launch_tables(const SetupArgs& sa, const double* omega, const double* gain,
                           const int* rev, float4* tables, ChannelCoef* coef, int* bad,
                           cudaStream_t s);

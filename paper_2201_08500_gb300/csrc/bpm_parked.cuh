@@ -30,10 +30,18 @@
 // barrier at its start and one between the parking and the second transform:
 // 8 block barriers a step.
 //
-// States of a step: [E0 in v, Eh parked] -> propagate E0 -> park E0, take Eh
-// -> propagate Eh -> [Eh in v, E0 parked] -> couple (reading E0 back) ->
-// [E0 in v, Eh parked].  Strang adds a coupling in the first state; fourth
-// order runs three (propagate both, couple) rounds after it.
+// The envelopes take turns: a step propagates the one in registers, swaps it
+// with the parked one, propagates that and couples in place, so the next step
+// begins with the other one.  The coupling touches the parked envelope and the
+// deformation row only where the crystal is (its extent in x over all rows): a
+// Bragg slab fills a tenth of the grid, and the L1 data path, which this march
+// keeps busiest (60 % of its cycles, the FP32 pipe 56 %), carries one park and
+// one unpark a step instead of four passes over an envelope.  Strang adds a
+// coupling before; fourth order runs three (propagate both, couple) rounds
+// after it.  us a step, before and after: 1024 channels of 8192 points 74.8 ->
+// 72.3, 4096 29.9 -> 29.0, 2048 13.85 -> 13.25, 1024 7.65 -> 7.26 (tables in
+// TMEM); Strang 512 x 4096 20.2 -> 18.2, 2048 10.25 -> 8.8; tables from L2
+// 1024 x 4096 40.7 -> 34.8.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -45,7 +53,9 @@ namespace bpm {
 
 // TMEM = true keeps each thread's propagator-table slice in tensor memory
 // (bpm_tmem.cuh, 128 columns per thread: 2 envelopes x 16 positions x hi/lo
-// float4) instead of reading it from L2 every step (one table set: SPLIT 1, 2).
+// float4) instead of reading it from L2 every step.  That is room for one set:
+// of the fourth order's two, the one of t dz, used twice a step; the other is
+// read from L2.
 // G channels per block (G x T threads; G > 1 at N = 1024, where a channel's 64
 // threads would leave half of each block's tensor-memory lanes unused): each
 // channel's T threads march their own channels with their own shared-memory
@@ -54,7 +64,6 @@ namespace bpm {
 template <int N, int SPLIT = 1, bool TMEM = false, bool WIDE = (N <= 4096), int G = 1>
 struct Parked {
   static_assert(SPLIT == 1 || SPLIT == 2 || SPLIT == 4, "splitting order");
-  static_assert(!TMEM || SPLIT != 4, "TMEM tables: one table set");
   using Gm = Geom<N>;
   static constexpr int T = Gm::T;
   static constexpr int S = Gm::S;
@@ -235,10 +244,10 @@ struct Parked {
     }
   }
 
-  // Table multiply of one envelope: 16 positions, hi/lo float4 each, from L2
-  // (gt) or from this thread's TMEM columns (tcol).
+  // Table multiply of one envelope: 16 positions, hi/lo float4 each, from this
+  // thread's TMEM columns (tcol) or, if there are none or gt is given, from L2.
   static BPM_DEV void multiply(float2 (&v)[16], const float4* gt, uint32_t tcol, int t) {
-    if constexpr (TMEM) {
+    if (TMEM && (SPLIT != 4 || !gt)) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         float4 tv[4];
@@ -335,77 +344,77 @@ struct Parked {
     }
   }
 
-  // [E0 in v, Eh parked] -> [Eh in v, E0 parked], both propagated (table set gt).
-  // Before: each thread's last accesses of p0 and ph were to its own slots.
-  // After: p0 and ph hold the parked E0 and (free) slots of Eh; other threads
-  // may still load from x.
-  static BPM_DEV void propagate_both(float2 (&v)[16], float2* x, float2* p0, float2* ph,
-                                     const float4* gt, uint32_t tcol, const float4* tw, int t) {
-    gsync();  // own-slot accesses of p0 / ph and loads of x are done
-    propagate(v, x, p0, gt, tcol, tw, t);  // p0 is free while E0 is in registers
-    park(v, p0, t);
-    unpark(v, ph, t);
-    gsync();  // x loads and the unparking of ph are done
-    propagate(v, x, ph, gt + N, tcol + 64u, tw, t);
+  // Park of envelope e (0: E0, 1: Eh), behind the exchange buffer x.
+  static BPM_DEV float2* park_of(float2* x, int e) { return x + (1 + e) * Pad<N>::kSlots; }
+
+  // Parks the envelope in v and takes the other one.
+  static BPM_DEV void swap_in(float2 (&v)[16], float2* x, int& held, int t) {
+    Parked::park(v, park_of(x, held), t);
+    held ^= 1;
+    unpark(v, park_of(x, held), t);
   }
 
-  // [Eh in v, E0 parked] -> coupling at z_n -> [E0 in v, Eh parked].
-  static BPM_DEV void couple_back(float2 (&v)[16], const float2* p0, float2* ph,
-                                  const float2* crow, const ChannelCoef& cf, int t) {
-    if constexpr (kWide) {
-      const float4* q0 = reinterpret_cast<const float4*>(p0);
-      float4* qh = reinterpret_cast<float4*>(ph);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {  // pair (2i, 2i+1)
-        const float4 w = q0[park_slot(t, i)];
-        float2 e0[2] = {make_float2(w.x, w.y), make_float2(w.z, w.w)};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float2 c = __ldg(crow + t + T * (2 * i + h));
-          if (c.x != 0.f || c.y != 0.f) couple_cell(e0[h], v[2 * i + h], c, cf);
-        }
-        qh[park_slot(t, i)] =
-            make_float4(v[2 * i].x, v[2 * i].y, v[2 * i + 1].x, v[2 * i + 1].y);
-        v[2 * i] = e0[0];
-        v[2 * i + 1] = e0[1];
+  // The two envelopes take turns in registers: `held` is the one in v, the
+  // other lies in its park and the park of `held` is free.  Propagates both
+  // (tables gt in L2; null: the set in TMEM) and leaves the other one in v.
+  // Before: each thread's last accesses of the parks were to its own slots.
+  // After: the same, and other threads may still load from x.
+  static BPM_DEV void propagate_both(float2 (&v)[16], float2* x, int& held, const float4* gt,
+                                     uint32_t tcol, const float4* tw, int t) {
+    if constexpr (N <= 1024) {
+      // one copy of the transform in the code: 7.45 -> 7.30 us a step of 1024
+      // channels (with it 2048 to 8192 points are 1 to 6 % slower)
+#pragma unroll 1
+      for (int j = 0; j < 2; ++j) {
+        gsync();  // own-slot accesses of the parks and loads of x are done
+        propagate(v, x, park_of(x, held), gt ? gt + held * N : gt, tcol + 64u * held, tw, t);
+        if (j == 0) swap_in(v, x, held, t);
       }
     } else {
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const float2 c = __ldg(crow + t + T * k);
-        float2 e0 = p0[k * T + t], eh = v[k];
-        if (c.x != 0.f || c.y != 0.f) couple_cell(e0, eh, c, cf);
-        ph[k * T + t] = eh;
-        v[k] = e0;
-      }
+      gsync();
+      propagate(v, x, park_of(x, held), gt ? gt + held * N : gt, tcol + 64u * held, tw, t);
+      swap_in(v, x, held, t);
+      gsync();  // x loads and the unparking are done
+      propagate(v, x, park_of(x, held), gt ? gt + held * N : gt, tcol + 64u * held, tw, t);
     }
   }
 
-  // [E0 in v, Eh parked] -> coupling at z_n, same state.
-  static BPM_DEV void couple_front(float2 (&v)[16], float2* ph, const float2* crow,
-                                   const ChannelCoef& cf, int t) {
+  // Coupling at z_n in place: the envelope in v stays there, and the parked one
+  // is read and written only where the crystal is.  Bit k of *mask: some of the
+  // cells T k + t of value k lie in the crystal's extent (the same for all
+  // threads); elsewhere nothing is loaded.  The row's loads go out together.
+  static BPM_DEV void couple(float2 (&v)[16], float2* parked_env, int held, const float2* crow,
+                             const ChannelCoef& cf, const unsigned* mask, int t) {
+    const unsigned m = *mask;
+    float2 c[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      c[k] = (m >> k) & 1u ? __ldg(crow + t + T * k) : make_float2(0.f, 0.f);
+    auto cell = [&](float2& in_v, float2& in_park, float2 ck) {
+      if (ck.x == 0.f && ck.y == 0.f) return;
+      float2 e0 = held ? in_park : in_v, eh = held ? in_v : in_park;
+      couple_cell(e0, eh, ck, cf);
+      in_v = held ? eh : e0;
+      in_park = held ? e0 : eh;
+    };
     if constexpr (kWide) {
-      float4* qh = reinterpret_cast<float4*>(ph);
+      float4* q = reinterpret_cast<float4*>(parked_env);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {  // pair (2i, 2i+1)
-        const float4 w = qh[park_slot(t, i)];
-        float2 eh[2] = {make_float2(w.x, w.y), make_float2(w.z, w.w)};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float2 c = __ldg(crow + t + T * (2 * i + h));
-          if (c.x != 0.f || c.y != 0.f) couple_cell(v[2 * i + h], eh[h], c, cf);
-        }
-        qh[park_slot(t, i)] = make_float4(eh[0].x, eh[0].y, eh[1].x, eh[1].y);
+        if (!((m >> (2 * i)) & 3u)) continue;
+        const float4 w = q[park_slot(t, i)];
+        float2 a = make_float2(w.x, w.y), b = make_float2(w.z, w.w);
+        cell(v[2 * i], a, c[2 * i]);
+        cell(v[2 * i + 1], b, c[2 * i + 1]);
+        q[park_slot(t, i)] = make_float4(a.x, a.y, b.x, b.y);
       }
     } else {
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
-        const float2 c = __ldg(crow + t + T * k);
-        if (c.x != 0.f || c.y != 0.f) {
-          float2 eh = ph[k * T + t];
-          couple_cell(v[k], eh, c, cf);
-          ph[k * T + t] = eh;
-        }
+        if (!((m >> k) & 1u)) continue;
+        float2 a = parked_env[k * T + t];
+        cell(v[k], a, c[k]);
+        parked_env[k * T + t] = a;
       }
     }
   }
@@ -435,14 +444,18 @@ struct Parked {
   static BPM_DEV void march_channel(const MarchArgs& A, int ch, unsigned char* smem, int t,
                                     uint32_t tcol = 0) {
     float2* x = reinterpret_cast<float2*>(smem);
-    float2* p0 = x + Pad<N>::kSlots;
-    float2* ph = p0 + Pad<N>::kSlots;
-    double* red = reinterpret_cast<double*>(ph + Pad<N>::kSlots);
+    double* red = reinterpret_cast<double*>(park_of(x, 2));
     const float4* gtab = A.tables + size_t(ch) * kTabs * 2 * N;
     // first order: the coupling coefficients are read from shared memory at
-    // each coupling instead of held in eight registers across the transforms
+    // each coupling instead of held in eight registers across the transforms;
+    // so is the crystal's extent (see couple)
     ChannelCoef* scf = reinterpret_cast<ChannelCoef*>(red + 32);
+    unsigned* mask = reinterpret_cast<unsigned*>(red + 40);
     if (SPLIT == 1 && t == 0) scf[0] = A.coef[ch];
+    if (t == 0) {
+      const int lo = __ldg(A.ext), hi = -__ldg(A.ext + 1);  // crystal cells [lo, hi)
+      *mask = lo == kExtNone ? 0u : (2u << ((hi - 1) / T)) - (1u << (lo / T));
+    }
     gsync();
     const ChannelCoef cfr = A.coef[size_t(ch) * kTabs];
     const ChannelCoef& cf = SPLIT == 1 ? scf[0] : cfr;
@@ -451,36 +464,40 @@ struct Parked {
     float2* eh = A.eh + size_t(ch) * N;
     if constexpr (TMEM) tmem_fill(gtab, tcol, t);
     float2 v[16];
+    int held = 0;
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = eh[t + T * k];
-    park(v, ph, t);
+    park(v, park_of(x, 1), t);
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = e0[t + T * k];
     for (int step = 0; step < A.n_steps; ++step) {
       const float2* crow = A.cfield + size_t(A.z0 + step) * N;
       if constexpr (SPLIT == 4) {
         const ChannelCoef cf1 = A.coef[size_t(ch) * 2 + 1];
-        couple_front(v, ph, crow, cf, t);
+        couple(v, park_of(x, held ^ 1), held, crow, cf, mask, t);
 #pragma unroll 1
         for (int j = 0; j < 3; ++j) {
-          propagate_both(v, x, p0, ph, gtab + (j == 1 ? 2 * N : 0), tcol, tw, t);
-          couple_back(v, p0, ph, crow, j == 2 ? cf : cf1, t);
+          propagate_both(v, x, held, j == 1 ? gtab + 2 * N : (TMEM ? nullptr : gtab), tcol, tw, t);
+          couple(v, park_of(x, held ^ 1), held, crow, j == 2 ? cf : cf1, mask, t);
         }
       } else {
-        if constexpr (SPLIT == 2) couple_front(v, ph, crow, cf, t);
-        propagate_both(v, x, p0, ph, gtab, tcol, tw, t);
-        couple_back(v, p0, ph, crow, cf, t);
+        if constexpr (SPLIT == 2) couple(v, park_of(x, held ^ 1), held, crow, cf, mask, t);
+        propagate_both(v, x, held, TMEM ? nullptr : gtab, tcol, tw, t);
+        couple(v, park_of(x, held ^ 1), held, crow, cf, mask, t);
       }
     }
-    double sa = 0.0, sb = 0.0;
+    // sums of |E|^2 of the envelope in v and of the parked one
+    float2 *fv = held ? eh : e0, *fp = held ? e0 : eh;
+    double sv = 0.0, sp = 0.0;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-      const float2 m = parked(ph, t, k);
-      e0[t + T * k] = v[k];
-      eh[t + T * k] = m;
-      sa += double(v[k].x) * v[k].x + double(v[k].y) * v[k].y;
-      sb += double(m.x) * m.x + double(m.y) * m.y;
+      const float2 m = parked(park_of(x, held ^ 1), t, k);
+      fv[t + T * k] = v[k];
+      fp[t + T * k] = m;
+      sv += double(v[k].x) * v[k].x + double(v[k].y) * v[k].y;
+      sp += double(m.x) * m.x + double(m.y) * m.y;
     }
+    double sa = held ? sp : sv, sb = held ? sv : sp;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       sa += __shfl_xor_sync(0xFFFFFFFFu, sa, off);

@@ -102,66 +102,90 @@ __device__ __forceinline__ dc tilted_propagator(double k, double Q2, double dz) 
   return dc{m * c, m * s};
 }
 
-// Crystal mask Pi(x_j, z_n) (the crystal's boundaries set the geometry, end of
-// Section 2): x_surface + z tan_psi <= x_j < x_end + z tan_psi and
-// z_begin <= z_n < z_end, with x_j = j dx, z_n = n dz.  Every product and sum is
-// rounded explicitly (no contraction) so that the decision is reproducible.
-__device__ __forceinline__ bool in_crystal(const SetupArgs& sa, int j, int n) {
-  const double x = __dmul_rn(double(j), sa.dx);
+// First cell j of a row whose x_j = j dx (rounded, so that the decision is
+// reproducible) is not below (END = false) or not under (END = true: !(x < b))
+// the bound b; sa.nx if none is.
+template <bool END>
+__device__ int first_cell(const SetupArgs& sa, double b) {
+  auto past = [&](int j) {
+    const double x = __dmul_rn(double(j), sa.dx);
+    return END ? !(x < b) : x >= b;
+  };
+  const double g = ceil(b / sa.dx);
+  int j = g >= 0.0 ? (g < double(sa.nx) ? int(g) : sa.nx) : 0;
+  while (j > 0 && past(j - 1)) --j;
+  while (j < sa.nx && !past(j)) ++j;
+  return j;
+}
+
+// Crystal cells [lo, hi) of a row at z_n = n dz from the crystal's boundaries
+// (they set the geometry, end of Section 2): x_surface + z tan_psi <= x_j <
+// x_end + z tan_psi and z_begin <= z_n < z_end.  Products and sums are rounded
+// explicitly (no contraction).
+__device__ int2 crystal_row(const SetupArgs& sa, int n) {
   const double z = __dmul_rn(double(n), sa.dz);
-  if (!(z >= sa.z_begin && z < sa.z_end)) return false;
+  if (!(z >= sa.z_begin && z < sa.z_end)) return make_int2(0, 0);
   const double shift = __dmul_rn(z, sa.tan_psi);
-  return x >= __dadd_rn(sa.x_surface, shift) && x < __dadd_rn(sa.x_end, shift);
+  const int lo = first_cell<false>(sa, __dadd_rn(sa.x_surface, shift));
+  const int hi = first_cell<true>(sa, __dadd_rn(sa.x_end, shift));
+  return lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
 }
 
-__global__ void deformation_kernel(SetupArgs sa, const double* __restrict__ u, float2* cfield) {
-  const long long plane = (long long)sa.nx * sa.ny;
-  const long long total = plane * sa.nz;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int j = int(i % sa.nx);
-    const bool in = sa.mask ? sa.mask[i] != 0 : in_crystal(sa, j, int(i / plane));
-    float2 c = make_float2(0.f, 0.f);
-    if (in) {
-      const double ph = u ? sa.h * u[i] : 0.0;
-      double s, co;
-      sincos(ph, &s, &co);
-      c = make_float2(float(co), float(s));
-    }
-    cfield[i] = c;
-  }
-}
-
-// Crystal extent of each deformation row (one block per row at a time).
-__global__ void crystal_span_kernel(const float2* __restrict__ cfield, int nx, long long rows,
-                                    int2* span) {
-  __shared__ int slo[32], shi[32];
-  for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
-    const float2* row = cfield + r * nx;
-    int lo = nx, hi = -1;
-    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-      const float2 c = row[x];
-      if (c.x != 0.f || c.y != 0.f) {
-        lo = min(lo, x);
-        hi = max(hi, x);
-      }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      lo = min(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, off));
-      hi = max(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, off));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      slo[threadIdx.x / 32] = lo;
-      shi[threadIdx.x / 32] = hi;
+// Deformation factor c = Pi exp(+i h u) of every row, with the rows' crystal
+// extents (span, 3D: the row pass loads c only there) or their union (ext =
+// {lo, -hi}, 2D: the parked march couples only there; starts at kExtNone).
+// FP64 only where there is crystal: a row's boundaries are found once instead
+// of tested in every cell, and vacuum is written without a look at u.
+// 2000 x 4096: 230 -> 71 us.
+constexpr int kDefRows = 8;
+__global__ void __launch_bounds__(256)
+    deformation_kernel(SetupArgs sa, const double* __restrict__ u, float2* cfield, int2* span,
+                       int* ext) {
+  __shared__ int slo[kDefRows], shi[kDefRows];
+  const long long rows = (long long)sa.nz * sa.ny;
+  const int pairs = sa.nx / 2;
+  for (long long r0 = (long long)blockIdx.x * kDefRows; r0 < rows;
+       r0 += (long long)gridDim.x * kDefRows) {
+    if (threadIdx.x < kDefRows) {
+      int2 b = make_int2(sa.nx, 0);  // a mask's extent is found with its cells
+      if (!sa.mask && r0 + threadIdx.x < rows) b = crystal_row(sa, int((r0 + threadIdx.x) / sa.ny));
+      slo[threadIdx.x] = b.x;
+      shi[threadIdx.x] = b.y;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < int(blockDim.x / 32); ++w) {
-        lo = min(lo, slo[w]);
-        hi = max(hi, shi[w]);
+    const int n_rows = int(min((long long)kDefRows, rows - r0));
+    for (int i = threadIdx.x; i < n_rows * pairs; i += blockDim.x) {
+      const int r = i / pairs, j = 2 * (i % pairs);
+      const size_t cell = size_t(r0 + r) * sa.nx + j;
+      float2 c[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        bool in;
+        if (sa.mask) {
+          in = sa.mask[cell + h] != 0;
+          if (in) {
+            atomicMin(&slo[r], j + h);
+            atomicMax(&shi[r], j + h + 1);
+          }
+        } else {
+          in = j + h >= slo[r] && j + h < shi[r];
+        }
+        if (in) {
+          double s = 0.0, co = 1.0;
+          if (u) sincos(sa.h * u[cell + h], &s, &co);
+          c[h] = make_float2(float(co), float(s));
+        }
       }
-      span[r] = hi < 0 ? make_int2(0, 0) : make_int2(lo, hi + 1);
+      *reinterpret_cast<float4*>(cfield + cell) = make_float4(c[0].x, c[0].y, c[1].x, c[1].y);
+    }
+    __syncthreads();
+    if (threadIdx.x < n_rows) {
+      const int lo = slo[threadIdx.x], hi = shi[threadIdx.x];
+      if (span) span[r0 + threadIdx.x] = lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
+      if (ext && lo < hi) {
+        atomicMin(ext, lo);
+        atomicMin(ext + 1, -hi);
+      }
     }
     __syncthreads();
   }
@@ -557,18 +581,14 @@ __global__ void __launch_bounds__(kIncThreads)
 }  // namespace
 
 cudaError_t launch_deformation(const SetupArgs& sa, const double* u_dev, float2* cfield,
-                               cudaStream_t s) {
-  const long long total = (long long)sa.nx * sa.ny * sa.nz;
-  long long blocks = (total + 255) / 256;
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  deformation_kernel<<<int(blocks), 256, 0, s>>>(sa, u_dev, cfield);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_crystal_span(const float2* cfield, int nx, long long rows, int2* span,
-                                cudaStream_t s) {
-  const long long blocks = rows < 152 * 16 ? rows : 152 * 16;
-  crystal_span_kernel<<<int(blocks), 256, 0, s>>>(cfield, nx, rows, span);
+                               int2* span, int* ext, cudaStream_t s) {
+  if (ext) {
+    const cudaError_t e = cudaMemsetAsync(ext, kExtNoneByte, 2 * sizeof(int), s);
+    if (e != cudaSuccess) return e;
+  }
+  const long long groups = ((long long)sa.ny * sa.nz + kDefRows - 1) / kDefRows;
+  deformation_kernel<<<unsigned(groups < 152 * 32 ? groups : 152 * 32), 256, 0, s>>>(sa, u_dev, cfield,
+                                                                                    span, ext);
   return cudaGetLastError();
 }
 

@@ -195,7 +195,7 @@ BPM_API bpm_status bpm_run_noalloc(const bpm_grid* grid, int n_channels,
 
   float2* e0 = static_cast<float2*>(e0_dev);
   float2* eh = static_cast<float2*>(eh_dev);
-  BPM_SCUDA(launch_deformation(sa, u_field_dev, cfield, st), "deformation kernel");
+  BPM_SCUDA(launch_deformation(sa, u_field_dev, cfield, nullptr, nullptr, st), "deformation kernel");
   BPM_SCUDA(launch_tables(sa, d_omega, gain, rev, tables, coef, flag, st), "tables kernel");
   BPM_SCUDA(launch_incident(sa, d_omega, d_weight, e0, eh, inc_norm,
                             reinterpret_cast<NormScratch*>(base + kOffNormParts), st), "incident kernel");
@@ -206,6 +206,7 @@ BPM_API bpm_status bpm_run_noalloc(const bpm_grid* grid, int n_channels,
   a.twiddle_t = nullptr;  // nx <= 4096: twiddles stay in registers
   a.twiddle_p = nullptr;
   a.cfield = cfield;
+  a.ext = nullptr;  // the forms launched here take the rows as they are
   a.e0 = e0;
   a.eh = eh;
   a.inc_norm = inc_norm;
