@@ -1325,37 +1325,41 @@ bpm_status enqueue_round(bpm_batch b, RoundSlot& r, int chunk) {
   };
   std::vector<Tmp> tmp;
   std::vector<int> steps(act.size());
+  const DeviceInfo& di = device_info();
+  const int sms = b->max_blocks > 0 ? std::min(b->max_blocks, di.sm_count) : di.sm_count;
+  int channels[kQueueCount] = {}, items[kQueueCount] = {};
+  for (int i : act) {
+    bpm_plan p = b->entries[i].plan;
+    const int q = batch_queue(p->grid.nx, p->grid.split_order);
+    const int G = batch_item_channels(p->grid.nx, p->grid.split_order);
+    // the small sizes of one order share a queue: count them by their own
+    const int c = G > 1 ? batch_single_queue(p->grid.nx, p->grid.split_order) : q;
+    channels[c] += p->n_ch;
+    items[c] += (p->n_ch + G - 1) / G;
+  }
   for (int k = 0; k < int(act.size()); ++k) {
     bpm_plan p = b->entries[act[k]].plan;
     const int n = p->grid.nx;
     steps[k] = std::min(chunk, p->grid.nz - p->z);
-    const int G = batch_item_channels(n, p->grid.split_order);
-    const int q = batch_queue(n, p->grid.split_order);
-    for (int c0 = 0; c0 < p->n_ch;) {
-      const int left = std::min(G, p->n_ch - c0);
-      int qs = q;
-      const bool single = G > 1 && batch_singles(n, p->grid.split_order, left, &qs);
-      const int take = single ? 1 : left;
+    int G = batch_item_channels(n, p->grid.split_order);
+    int q = batch_queue(n, p->grid.split_order);
+    if (G > 1) {
+      const int c = batch_single_queue(n, p->grid.split_order);
+      if (batch_singles(n, p->grid.split_order, channels[c], items[c], sms)) {
+        G = 1;
+        q = c;
+      }
+    }
+    for (int c0 = 0; c0 < p->n_ch; c0 += G) {
       Tmp t;
       t.it = BatchItem{k, c0, n, 0};
-      t.cost = double(steps[k]) * n * take * std::log2(double(n));
-      t.q = single ? qs : q;
+      t.cost = double(steps[k]) * n * std::min(G, p->n_ch - c0) * std::log2(double(n));
+      t.q = q;
       tmp.push_back(t);
-      c0 += take;
     }
   }
-  // launch rank of each queue: the longest items (Nx = 8192, every order) first,
-  // then 4096, 2048 and 1024, then the resident small-N queues
-  static constexpr int kOrder[kQueueCount] = {
-      kQueueTm8192,   kQueueTm8192s2, kQueueBig4,     kQueueTm4096,   kQueueTm4096s2,
-      kQueuePk4096s4, kQueueTm2048,   kQueueTm2048s2, kQueuePk2048s4, kQueueTm1024,
-      kQueuePk1024s4, kQueueQuad1024s2, kQueueSmall,  kQueueSmall2,   kQueueSmall4,
-      kQueueQuad512,  kQueueQuad512s2, kQueueQuad512s4, kQueueQuad256, kQueueQuad256s2,
-      kQueueQuad256s4};
-  int rank[kQueueCount];
-  for (int i = 0; i < kQueueCount; ++i) rank[kOrder[i]] = i;
-  std::stable_sort(tmp.begin(), tmp.end(), [&rank](const Tmp& x, const Tmp& y) {
-    return x.q != y.q ? rank[x.q] < rank[y.q] : x.cost > y.cost;
+  std::stable_sort(tmp.begin(), tmp.end(), [](const Tmp& x, const Tmp& y) {
+    return x.q != y.q ? x.q < y.q : x.cost > y.cost;
   });
   int cnt[kQueueCount] = {};
   for (auto& t : tmp) cnt[t.q]++;
@@ -1363,8 +1367,6 @@ bpm_status enqueue_round(bpm_batch b, RoundSlot& r, int chunk) {
   if (r.used) BPM_BCUDA(b, cudaEventSynchronize(r.free_ev), "staging reuse");
   for (int k = 0; k < int(act.size()); ++k) r.h_plans[k] = march_args(b->entries[act[k]].plan, steps[k]);
   for (size_t i = 0; i < tmp.size(); ++i) r.h_items[i] = tmp[i].it;
-  const DeviceInfo& di = device_info();
-  const int sms = b->max_blocks > 0 ? std::min(b->max_blocks, di.sm_count) : di.sm_count;
   BPM_BCUDA(b, cudaMemcpyAsync(r.d_plans, r.h_plans, sizeof(MarchArgs) * act.size(),
                                cudaMemcpyHostToDevice, b->stream), "upload round");
   BPM_BCUDA(b, cudaMemcpyAsync(r.d_items, r.h_items, sizeof(BatchItem) * tmp.size(),
@@ -1375,15 +1377,14 @@ bpm_status enqueue_round(bpm_batch b, RoundSlot& r, int chunk) {
   // blocks per SM: the Nx = 8192 items (the longest) first, then the smaller
   // ones; the idle tail is one item per queue.
   int off = 0;
-  for (int i = 0; i < kQueueCount; ++i) {
-    const int q = kOrder[i];
+  for (int q = 0; q < kQueueCount; ++q) {
     if (cnt[q] > 0)
       BPM_BCUDA(b, launch_batch(r.d_plans, r.d_items + off, cnt[q], r.d_counter + q, q,
                                 std::min(cnt[q], sms * batch_blocks_per_sm(q)), b->stream),
                 "batch kernel");
     off += cnt[q];
   }
-  const int n_big = cnt[kQueueTm8192] + cnt[kQueueTm8192s2] + cnt[kQueueBig4];
+  const int n_big = cnt[kQueueTm8192] + cnt[kQueueTm8192s2] + cnt[kQueueTm8192s4];
   const int n_small = int(tmp.size()) - n_big;
   BPM_BCUDA(b, cudaEventRecord(r.free_ev, b->stream), "round event");
   r.used = true;

@@ -2,15 +2,11 @@
 // plans (instances of different Nx, z-step counts and channel counts).
 //
 // Items are (plan, first channel) pairs sorted longest-first on the host.
-// Every block repeatedly takes the next item with an atomic counter and runs
-// the resident march of that item's transform size on G = 256 / T channels
-// (T = Nx/16 threads per channel): Nx = 256, 512, 1024, 2048, 4096 pack 16, 8,
-// 4, 2, 1 channels into the 256-thread block, each with its own shared-memory
-// slot (at most 196 KB).  Nx = 8192 needs 512 threads and runs in a sibling
-// kernel of the same structure, with the parked-envelope body (bpm_parked.cuh).
-// First-order items at Nx >= 1024 run in the tensor-memory kernels below;
-// second- and fourth-order items in their own instantiations of the two
-// kernels above (one queue per order and size class).  The counter lives in global memory and is
+// Every block repeatedly takes the next item with an atomic counter: at Nx >=
+// 1024 one channel in the parked form with tables in tensor memory; below, G =
+// 256 / T channels (T = Nx/16 threads each) of the resident form, and single
+// channels of what fills no such item with 8 T threads (bpm_quad.cuh).  One
+// queue per size, order and kind.  The counter lives in global memory and is
 // cleared before each launch; the queue never waits, so no block can hang.
 #include <cuda_runtime.h>
 
@@ -31,11 +27,8 @@ constexpr size_t item_smem() {
 
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 
-constexpr size_t kSmallSmem =
-    cmax(cmax(cmax(item_smem<256>(), item_smem<512>()), cmax(item_smem<1024>(), item_smem<2048>())),
-         item_smem<4096>());
-static_assert(Resident<4096, 1, 4>::smem_bytes() <= kSmallSmem &&
-                  Resident<256, 16, 4>::smem_bytes() <= kSmallSmem &&
+constexpr size_t kSmallSmem = cmax(item_smem<256>(), item_smem<512>());
+static_assert(Resident<256, 16, 4>::smem_bytes() <= kSmallSmem &&
                   Resident<256, 16, 2>::smem_bytes() <= kSmallSmem,
               "every order's resident slot fits the first-order bound");
 
@@ -59,40 +52,19 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     switch (item.n) {
       case 256: Resident<256, 16, SPLIT>::run_item(A, item.ch0, smem); break;
       case 512: Resident<512, 8, SPLIT>::run_item(A, item.ch0, smem); break;
-      case 1024: Resident<1024, 4, SPLIT>::run_item(A, item.ch0, smem); break;
-      case 2048: Resident<2048, 2, SPLIT>::run_item(A, item.ch0, smem); break;
-      case 4096: Resident<4096, 1, SPLIT>::run_item(A, item.ch0, smem); break;
       default: break;
     }
   }
 }
 
-template <int SPLIT>
-__global__ void __launch_bounds__(512, 1)
-    batch_kernel_8192(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
-                      int n_items, int* counter) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int s_item;
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-    __syncthreads();
-    const int it = s_item;
-    if (it >= n_items) break;
-    const BatchItem item = items[it];
-    if (item.n == 8192) Parked<8192, SPLIT>::run_item(plans[item.plan], item.ch0, smem);
-  }
-}
-
 // Body of the TMEM queues: first order in the narrow layout (fewer spills in
-// the work-queue kernel, measured faster), Strang in the layout of its
-// single-plan kernel (wide at N <= 4096).
+// the work-queue kernel, measured faster), the others in the layout of their
+// single-plan kernels (wide at N <= 4096).
 template <int N, int SPLIT>
-using TmBody = Parked<N, SPLIT, true, SPLIT == 2 && N <= 4096>;
+using TmBody = Parked<N, SPLIT, true, SPLIT != 1 && N <= 4096>;
 
-// First-order and Strang items at Nx = 2048, 4096, 8192 in the parked form
-// with the tables in tensor memory (Parked<N, SPLIT, true>, the fastest
-// single-plan form there): one channel per item, N/16 threads per block,
+// Items at Nx = 2048, 4096, 8192 in the parked form with tables in tensor
+// memory (Parked<N, SPLIT, true>, the fastest single-plan form there): one channel per item, N/16 threads per block,
 // 512/(N/16) blocks per SM; every block allocates its TMEM columns once and
 // frees them on exit.
 template <int N, int SPLIT>
@@ -120,17 +92,17 @@ __global__ void __launch_bounds__(N / 16, 512 / (N / 16))
   if (threadIdx.x / 32 == 0) tmem_dealloc<P::kCols>(s_tbase);
 }
 
-// First-order items at Nx = 1024 in the tensor-memory parked form with two
-// channels per 128-thread block (Parked<1024, 1, true, true, 2>, the fastest
+// Items at Nx = 1024 in the tensor-memory parked form with two channels per
+// 128-thread block (Parked<1024, SPLIT, true, true, 2>, the fastest
 // single-plan form there): each channel group of 64 threads takes its own
 // items (its own slot for the counter's answer, its own named barrier), so
 // the two groups march at independent phases; four blocks per SM fill the
 // SM's 512 TMEM columns.
-template <int N>
+template <int N, int SPLIT>
 __global__ void __launch_bounds__(2 * (N / 16), 512 / (2 * (N / 16)))
     batch_kernel_tm2(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
                      int n_items, int* counter) {
-  using P = Parked<N, 1, true, true, 2>;
+  using P = Parked<N, SPLIT, true, true, 2>;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item[2];
   __shared__ uint32_t s_tbase;
@@ -154,14 +126,12 @@ __global__ void __launch_bounds__(2 * (N / 16), 512 / (2 * (N / 16)))
   if (threadIdx.x / 32 == 0) tmem_dealloc<P::kCols>(s_tbase);
 }
 
-// Fourth-order items at Nx = 1024, 2048, 4096 in the parked form with both
-// table sets read from L2 (Parked<N, 4>, the fastest single-plan form there):
-// one channel per item, N/16 threads per block, 512/(N/16) blocks per SM.
-template <int N, int SPLIT>
-__global__ void __launch_bounds__(N / 16, 512 / (N / 16))
-    batch_kernel_pk(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
-                    int n_items, int* counter) {
-  using P = Parked<N, SPLIT>;
+// Fourth-order items at Nx = 1024 in the parked form with both table sets read
+// from L2, eight blocks per SM: as a single plan 25.1 us a step of 1024
+// channels, against 26.1 with two channels a block and one set in TMEM.
+__global__ void __launch_bounds__(64, 8)
+    batch_kernel_pk1024s4(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
+                          int n_items, int* counter) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
   for (;;) {
@@ -171,11 +141,11 @@ __global__ void __launch_bounds__(N / 16, 512 / (N / 16))
     const int it = s_item;
     if (it >= n_items) break;
     const BatchItem item = items[it];
-    P::run_item(plans[item.plan], item.ch0, smem);
+    Parked<1024, 4>::march_channel(plans[item.plan], item.ch0, smem, threadIdx.x);
   }
 }
 
-// Single channels at Nx <= 1024 with 8 Nx/16 threads each (bpm_quad.cuh).
+// Single channels at Nx <= 512 with 8 Nx/16 threads each (bpm_quad.cuh).
 template <int N, int SPLIT>
 __global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>::kThreads)
     batch_kernel_quad(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
@@ -195,31 +165,29 @@ __global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>
 
 }  // namespace
 
-// A resident item takes the time of a full one however few channels it has
-// (us a step: 256 points 2.9, 512 points 4.7; Strang 4.4, 5.8, 1024 points
-// 5.65; fourth order 10.3, 15.6), a single channel of the other form 0.25,
-// 0.65; 0.275, 0.70, 1.97; 0.85, 2.29 of an SM's time.
-bool batch_singles(int n, int split_order, int left, int* queue) {
-  int most = 0;
-  if (split_order == 1) {
-    most = n == 256 ? 11 : n == 512 ? 7 : 0;
-    *queue = n == 256 ? kQueueQuad256 : kQueueQuad512;
-  } else if (split_order == 2) {
-    most = n == 256 ? 15 : n == 512 ? 8 : n == 1024 ? 2 : 0;
-    *queue = n == 256 ? kQueueQuad256s2 : n == 512 ? kQueueQuad512s2 : kQueueQuad1024s2;
-  } else {
-    most = n == 256 ? 12 : n == 512 ? 6 : 0;
-    *queue = n == 256 ? kQueueQuad256s4 : kQueueQuad512s4;
-  }
-  return left <= most;
+// A resident item takes an SM for the time of a full one however few channels
+// it has (us a step, first order, Strang, fourth order: 256 points 2.9, 4.4,
+// 10.3; 512 points 4.7, 5.8, 15.6), a channel of the other form its share of
+// one (0.25, 0.275, 0.85; 0.65, 0.70, 2.29).  One kind for the whole round: the
+// queues run one after the other.
+bool batch_singles(int n, int split_order, int channels, int items, int sms) {
+  if (n > 512 || sms < 1) return false;
+  const int i = n == 256 ? 0 : 1, o = split_order == 1 ? 0 : split_order == 2 ? 1 : 2;
+  static constexpr double each[2][3] = {{0.25, 0.275, 0.85}, {0.65, 0.70, 2.29}};
+  static constexpr double full[2][3] = {{2.9, 4.4, 10.3}, {4.7, 5.8, 15.6}};
+  return each[i][o] * ((channels + sms - 1) / sms) < full[i][o] * ((items + sms - 1) / sms);
+}
+
+int batch_single_queue(int n, int split_order) {
+  if (split_order == 1) return n == 256 ? kQueueQuad256 : kQueueQuad512;
+  if (split_order == 2) return n == 256 ? kQueueQuad256s2 : kQueueQuad512s2;
+  return n == 256 ? kQueueQuad256s4 : kQueueQuad512s4;
 }
 
 int batch_group(int n) { return n == 8192 ? 1 : kSmallThreads / (n / 16); }
 
 int batch_item_channels(int n, int split_order) {
-  const bool parked = (split_order <= 2 && n >= 2048) || (split_order == 1 && n == 1024) ||
-                      (split_order == 4 && n >= 1024 && n <= 4096);
-  return parked ? 1 : batch_group(n);
+  return n >= 1024 ? 1 : batch_group(n);  // parked forms from 1024 points on
 }
 
 int batch_queue(int n, int split_order) {
@@ -231,15 +199,16 @@ int batch_queue(int n, int split_order) {
     return kQueueSmall;
   }
   if (split_order == 4) {
-    if (n == 8192) return kQueueBig4;
-    if (n == 4096) return kQueuePk4096s4;
-    if (n == 2048) return kQueuePk2048s4;
+    if (n == 8192) return kQueueTm8192s4;
+    if (n == 4096) return kQueueTm4096s4;
+    if (n == 2048) return kQueueTm2048s4;
     if (n == 1024) return kQueuePk1024s4;
     return kQueueSmall4;
   }
   if (n == 8192) return kQueueTm8192s2;
   if (n == 4096) return kQueueTm4096s2;
   if (n == 2048) return kQueueTm2048s2;
+  if (n == 1024) return kQueueTm1024s2;
   return kQueueSmall2;
 }
 
@@ -247,11 +216,12 @@ int batch_blocks_per_sm(int queue) {
   switch (queue) {
     case kQueueTm4096:
     case kQueueTm4096s2:
-    case kQueuePk4096s4: return 2;
+    case kQueueTm4096s4: return 2;
     case kQueueTm2048:
     case kQueueTm2048s2:
-    case kQueuePk2048s4:
-    case kQueueTm1024: return 4;
+    case kQueueTm2048s4:
+    case kQueueTm1024:
+    case kQueueTm1024s2: return 4;
     case kQueuePk1024s4: return 8;
     case kQueueQuad256:
     case kQueueQuad256s2:
@@ -272,11 +242,12 @@ void tm_launch(const MarchArgs* plans, const BatchItem* items, int n_items, int*
       plans, items, n_items, counter);
 }
 
-template <int N, int SPLIT>
-void pk_launch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
-               int blocks, cudaStream_t s) {
-  batch_kernel_pk<N, SPLIT><<<blocks, N / 16, Parked<N, SPLIT>::smem_bytes(), s>>>(
-      plans, items, n_items, counter);
+template <int SPLIT>
+void tm2_launch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
+                int blocks, cudaStream_t s) {
+  batch_kernel_tm2<1024, SPLIT>
+      <<<blocks, 128, Parked<1024, SPLIT, true, true, 2>::smem_bytes(), s>>>(plans, items, n_items,
+                                                                             counter);
 }
 
 template <int N, int SPLIT>
@@ -292,10 +263,11 @@ cudaError_t tm_attr() {
                               int(TmBody<N, SPLIT>::smem_bytes()));
 }
 
-template <int N, int SPLIT>
-cudaError_t pk_attr() {
-  return cudaFuncSetAttribute(batch_kernel_pk<N, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(Parked<N, SPLIT>::smem_bytes()));
+template <int SPLIT>
+cudaError_t tm2_attr() {
+  return cudaFuncSetAttribute(batch_kernel_tm2<1024, SPLIT>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              int(Parked<1024, SPLIT, true, true, 2>::smem_bytes()));
 }
 
 }  // namespace
@@ -303,7 +275,6 @@ cudaError_t pk_attr() {
 cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
                          int queue, int blocks, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  const size_t big_smem = Parked<8192, 4>::smem_bytes();
   switch (queue) {
     case kQueueTm8192: tm_launch<8192, 1>(plans, items, n_items, counter, blocks, s); break;
     case kQueueTm4096: tm_launch<4096, 1>(plans, items, n_items, counter, blocks, s); break;
@@ -311,12 +282,14 @@ cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_i
     case kQueueTm8192s2: tm_launch<8192, 2>(plans, items, n_items, counter, blocks, s); break;
     case kQueueTm4096s2: tm_launch<4096, 2>(plans, items, n_items, counter, blocks, s); break;
     case kQueueTm2048s2: tm_launch<2048, 2>(plans, items, n_items, counter, blocks, s); break;
-    case kQueuePk4096s4: pk_launch<4096, 4>(plans, items, n_items, counter, blocks, s); break;
-    case kQueuePk2048s4: pk_launch<2048, 4>(plans, items, n_items, counter, blocks, s); break;
-    case kQueuePk1024s4: pk_launch<1024, 4>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm1024:
-      batch_kernel_tm2<1024><<<blocks, 128, Parked<1024, 1, true, true, 2>::smem_bytes(), s>>>(
-          plans, items, n_items, counter);
+    case kQueueTm8192s4: tm_launch<8192, 4>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueTm4096s4: tm_launch<4096, 4>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueTm2048s4: tm_launch<2048, 4>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueTm1024: tm2_launch<1>(plans, items, n_items, counter, blocks, s); break;
+    case kQueueTm1024s2: tm2_launch<2>(plans, items, n_items, counter, blocks, s); break;
+    case kQueuePk1024s4:
+      batch_kernel_pk1024s4<<<blocks, 64, Parked<1024, 4>::smem_bytes(), s>>>(plans, items, n_items,
+                                                                              counter);
       break;
     case kQueueSmall:
       batch_kernel<1><<<blocks, kSmallThreads, kSmallSmem, s>>>(plans, items, n_items, counter);
@@ -327,14 +300,10 @@ cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_i
     case kQueueSmall4:
       batch_kernel<4><<<blocks, kSmallThreads, kSmallSmem, s>>>(plans, items, n_items, counter);
       break;
-    case kQueueBig4:
-      batch_kernel_8192<4><<<blocks, 512, big_smem, s>>>(plans, items, n_items, counter);
-      break;
     case kQueueQuad256: quad_launch<256, 1>(plans, items, n_items, counter, blocks, s); break;
     case kQueueQuad512: quad_launch<512, 1>(plans, items, n_items, counter, blocks, s); break;
     case kQueueQuad256s2: quad_launch<256, 2>(plans, items, n_items, counter, blocks, s); break;
     case kQueueQuad512s2: quad_launch<512, 2>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueQuad1024s2: quad_launch<1024, 2>(plans, items, n_items, counter, blocks, s); break;
     case kQueueQuad256s4: quad_launch<256, 4>(plans, items, n_items, counter, blocks, s); break;
     case kQueueQuad512s4: quad_launch<512, 4>(plans, items, n_items, counter, blocks, s); break;
     default:
@@ -344,17 +313,16 @@ cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_i
 }
 
 cudaError_t batch_set_attributes() {
-  const int small = int(kSmallSmem), big = int(Parked<8192, 4>::smem_bytes());
+  const int small = int(kSmallSmem);
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t r[] = {cudaFuncSetAttribute(batch_kernel<1>, attr, small),
                      cudaFuncSetAttribute(batch_kernel<2>, attr, small),
                      cudaFuncSetAttribute(batch_kernel<4>, attr, small),
-                     cudaFuncSetAttribute(batch_kernel_8192<4>, attr, big),
                      tm_attr<8192, 1>(), tm_attr<4096, 1>(), tm_attr<2048, 1>(),
                      tm_attr<8192, 2>(), tm_attr<4096, 2>(), tm_attr<2048, 2>(),
-                     pk_attr<4096, 4>(), pk_attr<2048, 4>(), pk_attr<1024, 4>(),
-                     cudaFuncSetAttribute(batch_kernel_tm2<1024>, attr,
-                                          int(Parked<1024, 1, true, true, 2>::smem_bytes()))};
+                     tm_attr<8192, 4>(), tm_attr<4096, 4>(), tm_attr<2048, 4>(),
+                     tm2_attr<1>(), tm2_attr<2>(),
+                     cudaFuncSetAttribute(batch_kernel_pk1024s4, attr, int(Parked<1024, 4>::smem_bytes()))};
   for (cudaError_t e : r)
     if (e != cudaSuccess) return e;
   return cudaSuccess;

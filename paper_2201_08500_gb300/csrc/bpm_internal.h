@@ -117,34 +117,29 @@ struct BatchItem {
 // queues (longest items first within each) and launches the queues back to
 // back, the Nx = 8192 queues of every order first, then 4096, 2048, 1024 and
 // the resident small-N queues (enqueue_round in bpm_api.cu):
+// Nx >= 1024: parked form with tables in tensor memory (fourth order: one set
+// of two), 1, 2 and 4 blocks per SM at 8192, 4096 and below, at 1024 two
+// channels a block (fourth order: tables from L2, 8 blocks per SM); s2: Strang,
+// s4: fourth order.
 enum BatchQueue {
-  kQueueTm8192 = 0,  // first order, Nx = 8192: parked form, TMEM tables
-  kQueueTm4096,      // first order, Nx = 4096: parked form, TMEM tables, 2 blocks / SM
-  kQueueTm2048,      // first order, Nx = 2048: parked form, TMEM tables, 4 blocks / SM
-  kQueueSmall,       // first order, Nx <= 512: resident form, G channels per block
-  kQueueSmall2,      // Strang, Nx <= 1024: resident form
-  kQueueBig4,        // fourth order, Nx = 8192: parked form, L2 tables (two sets)
-  kQueueSmall4,      // fourth order, Nx <= 512: resident form, L2 tables (two sets)
-  kQueueTm8192s2,    // Strang, Nx = 8192: parked form, TMEM tables
-  kQueueTm4096s2,    // Strang, Nx = 4096: parked form, TMEM tables, 2 blocks / SM
-  kQueueTm2048s2,    // Strang, Nx = 2048: parked form, TMEM tables, 4 blocks / SM
-  kQueuePk4096s4,    // fourth order, Nx = 4096: parked form, L2 tables, 2 blocks / SM
-  kQueuePk2048s4,    // fourth order, Nx = 2048: parked form, L2 tables, 4 blocks / SM
-  kQueuePk1024s4,    // fourth order, Nx = 1024: parked form, L2 tables, 8 blocks / SM
-  kQueueTm1024,      // first order, Nx = 1024: parked form, TMEM tables, two channels a
-                     // block, 4 blocks / SM
-  // single channels at Nx <= 512 (Strang: 1024): 8 Nx/16 threads a channel (bpm_quad.cuh)
-  kQueueQuad256, kQueueQuad512,
-  kQueueQuad256s2, kQueueQuad512s2, kQueueQuad1024s2,
-  kQueueQuad256s4, kQueueQuad512s4,
-  kQueueCount
+  kQueueTm8192 = 0, kQueueTm8192s2, kQueueTm8192s4,
+  kQueueTm4096, kQueueTm4096s2, kQueueTm4096s4,
+  kQueueTm2048, kQueueTm2048s2, kQueueTm2048s4,
+  kQueueTm1024, kQueueTm1024s2, kQueuePk1024s4,
+  // Nx <= 512: resident form, G channels per block (one queue per order)
+  kQueueSmall, kQueueSmall2, kQueueSmall4,
+  // single channels at Nx <= 512: 8 Nx/16 threads a channel (bpm_quad.cuh)
+  kQueueQuad512, kQueueQuad512s2, kQueueQuad512s4,
+  kQueueQuad256, kQueueQuad256s2, kQueueQuad256s4,
+  kQueueCount  // in launch order: the longest items first
 };
 int batch_group(int n);                               // channels per block of the resident kernels
 int batch_item_channels(int n, int split_order);      // channels per item
 int batch_queue(int n, int split_order);
-// Items of a plan's last `left` channels (fewer than an item's channels, or a
-// full item): singles in queue *queue (true) or one resident item.
-bool batch_singles(int n, int split_order, int left, int* queue);
+// Whether a round's `channels` channels of plans of this size and order, `items`
+// resident items, run as single channels instead, and the queue of those.
+bool batch_singles(int n, int split_order, int channels, int items, int sms);
+int batch_single_queue(int n, int split_order);
 int batch_blocks_per_sm(int queue);
 cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
                          int queue, int blocks, cudaStream_t s);

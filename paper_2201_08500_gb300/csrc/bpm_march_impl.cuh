@@ -11,20 +11,25 @@
 namespace bpm {
 
 // Per-channel march body of a launch form: FORM 0 the register-resident form
-// for N <= 4096 and the parked-envelope form for N = 8192; FORM 1 the L2-table
+// for N <= 4096, and that of FORM 3 at N = 8192; FORM 1 the L2-table
 // resident form; FORM 2 the parked form at N <= 4096; FORM 3 the parked form
-// with the tables in tensor memory (at N = 1024 two channels a block).
+// with the tables in tensor memory (at N = 1024 two channels a block).  The
+// fourth order's parked forms (FORM 2 at N = 2048 and 4096, FORM 0 at 8192) keep
+// the table set that is used twice a step in tensor memory: against both sets
+// from L2, 512 channels of 4096 points 64.7 -> 55.2 us a step, of 2048 27.6 ->
+// 26.6, 304 of 8192 71.8 -> 69.1.  At 1024, where a TMEM block has two
+// channels, both from L2 is faster (25.1 against 26.1).
 template <int N, int G, int SPLIT, int FORM>
 struct MarchBody {
   using type = Resident<N, G, SPLIT, FORM == 1>;
 };
 template <int SPLIT>
 struct MarchBody<8192, 1, SPLIT, 0> {
-  using type = Parked<8192, SPLIT>;
+  using type = Parked<8192, SPLIT, true>;
 };
 template <int N, int SPLIT>
 struct MarchBody<N, 1, SPLIT, 2> {
-  using type = Parked<N, SPLIT>;
+  using type = Parked<N, SPLIT, SPLIT == 4 && N != 1024>;
 };
 template <int N, int SPLIT>
 struct MarchBody<N, 1, SPLIT, 3> {

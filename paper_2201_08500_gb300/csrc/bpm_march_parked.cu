@@ -48,7 +48,7 @@ cudaError_t launch_march_parked(int n, int form, int blocks, const MarchArgs& a,
     if (n == 8192) return launch_one<8192, 1, 2, 3>(blocks, a, s);
     return cudaErrorInvalidValue;
   }
-  if (form == 2 && a.split_order == 4) {  // fourth order: two table sets from L2
+  if (form == 2 && a.split_order == 4) {  // fourth order (one table set in TMEM at N >= 2048)
     if (n == 1024) return launch_one<1024, 1, 4, 2>(blocks, a, s);
     if (n == 2048) return launch_one<2048, 1, 4, 2>(blocks, a, s);
     if (n == 4096) return launch_one<4096, 1, 4, 2>(blocks, a, s);

@@ -542,11 +542,6 @@ struct Parked {
         march_channel(A, ch, gsmem, t);
     }
   }
-
-  static BPM_DEV void run_item(const MarchArgs& A, int ch0, unsigned char* smem) {
-    static_assert(!TMEM && G == 1, "work-queue items: one channel a block, tables from L2");
-    if (ch0 < A.n_ch) march_channel(A, ch0, smem, threadIdx.x);
-  }
 };
 
 }  // namespace bpm

@@ -29,12 +29,14 @@ def test_few_channels_give_the_resident_forms_bits(nx, n_ch, maxg, order):
             assert np.array_equal(a, b)
 
 
-def test_work_queue_singles_and_full_items_give_the_plans_bits():
-    """Plans of small grids in one batch: full resident items and the remainders
-    on either side of the line to single channels, each as marched alone."""
+@pytest.mark.parametrize("sms", [0, 4])
+def test_work_queue_singles_and_full_items_give_the_plans_bits(sms):
+    """Plans of small grids in one batch, on either side of the line between
+    single channels and resident items (on four SMs the larger counts fill
+    these), each as marched alone."""
     ws = []
-    for nx, order, counts in ((256, 1, (1, 27, 28)), (256, 2, (31,)), (256, 4, (12, 13)),
-                              (512, 1, (1, 15, 16)), (512, 2, (9,)), (512, 4, (6, 15)),
+    for nx, order, counts in ((256, 1, (1, 64)), (256, 2, (31,)), (256, 4, (61, 3)),
+                              (512, 1, (1, 15, 40)), (512, 2, (9,)), (512, 4, (6, 32)),
                               (1024, 2, (2, 7))):
         for n_ch in counts:
             w = deformed_small(nx, nz=20 + n_ch, n_ch=n_ch, seed=n_ch)
@@ -48,6 +50,7 @@ def test_work_queue_singles_and_full_items_give_the_plans_bits():
         want.append((p.e0(), p.eh(), p.reflectivity()[0]))
         p.close()
     b = bpm.Batch()
+    b.set_max_blocks(sms)
     plans = [bpm.plan_from_workload(w) for w in ws]
     for p in plans:
         b.submit(p)
