@@ -266,7 +266,10 @@ typedef struct {
 } bpm_launch;
 
 /* The plan's launch form (chosen at creation: the tuned form of its shape if
- * bpm_tune or bpm_tune_load provided one, else the default).  Errors: INVALID_ARG. */
+ * bpm_tune or bpm_tune_load provided one, else the default).  A plan with
+ * neither a tuned nor a forced form marches in the form that its size, order
+ * and channel count call for, and the default is only what bpm_set_launch
+ * starts from; bpm_get_stats describes what ran.  Errors: INVALID_ARG. */
 BPM_API bpm_status bpm_get_launch(bpm_plan plan, bpm_launch* out);
 
 /* Forces a launch form for later bpm_run calls (ms is ignored).

@@ -269,6 +269,9 @@ struct bpm_plan_s {
   unsigned char* mask = nullptr;  // caller's crystal shape [nz][ny][nx] (plan-owned copy) or null
   size_t bytes = 0;               // device bytes owned by the plan
 
+  // launch form: tuned or forced (chosen), else the base of bpm_set_launch, and
+  // bpm_run takes what march_default_form says
+  bool chosen = false;
   int group = 1, blocks = 0;
   int form = 0;  // march form: 0 tables in shared memory, 1 tables in L2 (two blocks / SM)
   int row_threads = 256;  // 3D row pass tile: 256 or 512 threads
@@ -359,23 +362,27 @@ bool launch_valid(const bpm_grid& g, int form, int group, int row_threads) {
   return form == 1 && g.split_order == 1 && march_l2_supported(g.nx, group);
 }
 
-// Derived launch quantities of the plan's form (2D: the march kernel's
-// geometry; 3D plans run two passes a step, whose grids the passes size
-// themselves, so only channels_per_block is set).
-void apply_launch(bpm_plan p) {
-  p->blocks = (p->n_ch + p->group - 1) / p->group;
-  p->stats.channels_per_block = p->group;
+// Blocks and statistics of a launch form (2D: the march kernel's geometry; 3D
+// plans run two passes a step, whose grids the passes size themselves, so only
+// channels_per_block is set).
+void apply_launch(bpm_plan p, int form, int group) {
+  p->blocks = (p->n_ch + group - 1) / group;
+  p->stats.channels_per_block = group;
   if (p->grid.dims == 3) {
     p->stats.threads_per_channel = 0;
     p->stats.blocks = 0;
     p->stats.smem_bytes = 0;
     return;
   }
-  p->stats.threads_per_channel = march_threads_per_channel(p->grid.nx);
+  const int nx = p->grid.nx;
+  const bool quad = form == 0 && group == 1 &&
+                    march_quad_use(nx, p->grid.split_order, p->n_ch, device_info().sm_count);
+  p->stats.threads_per_channel = quad ? 8 * (nx / 16) : march_threads_per_channel(nx);
   p->stats.blocks = p->blocks;
-  p->stats.smem_bytes = int(p->form == 1   ? march_l2_smem_bytes(p->grid.nx, p->group)
-                            : p->form >= 2 ? march_parked_smem_bytes(p->grid.nx, p->form)
-                                           : march_smem_bytes(p->grid.nx, p->group));
+  p->stats.smem_bytes = int(quad        ? march_quad_smem_bytes(nx)
+                            : form == 1 ? march_l2_smem_bytes(nx, group)
+                            : form >= 2 ? march_parked_smem_bytes(nx, form)
+                                        : march_smem_bytes(nx, group));
 }
 
 size_t plan_bytes(const bpm_grid& g, int n_ch) {
@@ -568,12 +575,13 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
     auto it = g_tune.find(tune_key(g, n_channels));
     if (it != g_tune.end() &&
         launch_valid(g, it->second.form, it->second.group, it->second.row_threads)) {
+      p->chosen = true;
       p->form = it->second.form;
       p->group = it->second.group;
       p->row_threads = it->second.row_threads;
     }
   }
-  apply_launch(p.get());
+  apply_launch(p.get(), p->form, p->group);
   p->bytes = plan_bytes(g, n_channels);
   *out = p.release();
   return BPM_OK;
@@ -804,13 +812,16 @@ BPM_API bpm_status bpm_run(bpm_plan p, int n_steps) {
   int launches = 0, march_launches = 0;
   if (p->timing) BPM_CUDA(p, cudaEventRecord(p->ev0, p->stream), "timing event");
   if (p->grid.dims == 2) {
-    if (p->form == 1 && a.split_order == 1)
-      BPM_CUDA(p, launch_march_l2(p->grid.nx, p->group, p->blocks, a, p->stream), "march kernel");
-    else if ((p->form == 2 && a.split_order != 2) || (p->form == 3 && a.split_order <= 2))
-      BPM_CUDA(p, launch_march_parked(p->grid.nx, p->form, p->blocks, a, p->stream),
-               "march kernel");
+    int form = p->form, group = p->group;
+    if (!p->chosen)
+      march_default_form(p->grid.nx, a.split_order, p->n_ch, device_info().sm_count, &form, &group);
+    apply_launch(p, form, group);
+    if (form == 1 && a.split_order == 1)
+      BPM_CUDA(p, launch_march_l2(p->grid.nx, group, p->blocks, a, p->stream), "march kernel");
+    else if ((form == 2 && a.split_order != 2) || (form == 3 && a.split_order <= 2))
+      BPM_CUDA(p, launch_march_parked(p->grid.nx, form, p->blocks, a, p->stream), "march kernel");
     else
-      BPM_CUDA(p, launch_march(p->grid.nx, p->group, p->blocks, a, p->stream), "march kernel");
+      BPM_CUDA(p, launch_march(p->grid.nx, group, p->blocks, a, p->stream), "march kernel");
     march_launches = 1;
   } else if (n_steps > 0) {
     Pass3DArgs pa;
@@ -988,10 +999,11 @@ BPM_API bpm_status bpm_set_launch(bpm_plan p, const bpm_launch* f) {
   if (!p || !f) return fail(p, BPM_ERR_INVALID_ARG, "null argument");
   if (!launch_valid(p->grid, f->form, f->channels_per_block, f->row_threads))
     return fail(p, BPM_ERR_INVALID_ARG, "launch form not available for this plan");
+  p->chosen = true;
   p->form = f->form;
   p->group = f->channels_per_block;
   p->row_threads = f->row_threads;
-  apply_launch(p);
+  apply_launch(p, p->form, p->group);
   return BPM_OK;
 }
 

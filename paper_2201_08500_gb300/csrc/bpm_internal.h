@@ -160,11 +160,13 @@ cudaError_t time_set_attributes();
 int march_threads_per_channel(int n);
 int march_max_group(int n);
 size_t march_smem_bytes(int n, int group);
+void march_default_form(int n, int split_order, int n_ch, int sms, int* form, int* group);
 cudaError_t launch_march(int n, int group, int blocks, const MarchArgs& a, cudaStream_t s);
 cudaError_t launch_march_strang(int n, int group, int blocks, const MarchArgs& a, cudaStream_t s);
 // The march with 8 n/16 threads a channel (bpm_march_quad.cu), n <= 1024, every
 // order: launch_march takes it for one channel a block where it is the faster.
 bool march_quad_use(int n, int split_order, int n_ch, int sms);
+size_t march_quad_smem_bytes(int n);
 cudaError_t launch_march_quad(int n, const MarchArgs& a, cudaStream_t s);
 // Second form of the first-order march: propagator tables and stage twiddles
 // read from L2 instead of shared memory / registers, at most 128 registers, so

@@ -37,6 +37,49 @@ int march_max_group(int n) {
   }
 }
 
+// Form and channels per block of a plan that names none, over 1 ... 2500
+// channels and 152 SMs (us a step, this form against the next best):
+//  * 256, 512 points: one channel a block while march_quad_use holds (1.45
+//    against 4.6 at 230 channels of 512), then at 256 sixteen (2.9 against 3.9
+//    at 2432);
+//  * 1024: one channel up to one an SM, fourth order and Strang up to two (1.8
+//    against 3.0 at 152 channels, 10.8 against 13.2 at 304); beyond, TMEM
+//    tables, two channels a block (3.0 against 3.6 at 230, 16.7 against 19.1 at
+//    2500), fourth order the parked form (18.7 against 23 at 611);
+//  * 2048: TMEM tables (4.06 against 4.41 at 152, 14.1 against 16.4 at 1024);
+//    fourth order the parked form beyond two channels an SM (21.4 against 29.2
+//    at 456, but 16.4 against 16.1 at 304);
+//  * 4096: the resident form up to one channel an SM (5.1 against 5.4), then
+//    TMEM tables (8.8 against 9.8 at 230, 30.7 against 37.4 at 1024), fourth
+//    order parked (28.3 against 34.2 at 230);
+//  * 8192: TMEM tables (form 0 is the same kernel).
+void march_default_form(int n, int split_order, int n_ch, int sms, int* form, int* group) {
+  *form = 0;
+  *group = 1;
+  const int o = split_order;
+  switch (n) {
+    case 256:
+      if (!march_quad_use(n, o, n_ch, sms)) *group = march_max_group(n);
+      break;
+    case 1024:
+      if (n_ch > (o == 1 ? sms : 2 * sms)) {
+        *form = o == 4 ? 2 : 3;
+        *group = o == 4 ? 1 : 2;
+      }
+      break;
+    case 2048:
+      if (o != 4)
+        *form = 3;
+      else if (n_ch > 2 * sms)
+        *form = 2;
+      break;
+    case 4096:
+      if (n_ch > sms) *form = o == 4 ? 2 : 3;
+      break;
+    default: break;
+  }
+}
+
 size_t march_smem_bytes(int n, int group) {
 #define BPM_SMEM_CASE(NN, GG) \
   if (n == NN && group == GG) return MarchBody<NN, GG, 1, 0>::type::smem_bytes();

@@ -37,9 +37,9 @@ struct MarchBody<N, 1, SPLIT, 3> {
 };
 // N = 1024: two channels of 64 threads per block, so that a block's 128
 // tensor-memory lanes all hold tables (four blocks of 128 columns per SM).
-template <>
-struct MarchBody<1024, 2, 1, 3> {
-  using type = Parked<1024, 1, true, true, 2>;
+template <int SPLIT>
+struct MarchBody<1024, 2, SPLIT, 3> {
+  using type = Parked<1024, SPLIT, true, true, 2>;
 };
 
 // Resident blocks per SM the form is compiled for (128 registers unless 1).

@@ -35,7 +35,7 @@ cudaError_t march_set_attributes_parked() {
                      attr_one<2048, 1, 2, 3>(), attr_one<4096, 1, 2, 3>(),
                      attr_one<8192, 1, 2, 3>(), attr_one<1024, 1, 4, 2>(),
                      attr_one<2048, 1, 4, 2>(), attr_one<4096, 1, 4, 2>(),
-                     attr_one<1024, 2, 1, 3>()};
+                     attr_one<1024, 2, 1, 3>(), attr_one<1024, 2, 2, 3>()};
   for (cudaError_t x : r)
     if (x != cudaSuccess) e = x;
   return e;
@@ -43,6 +43,7 @@ cudaError_t march_set_attributes_parked() {
 
 cudaError_t launch_march_parked(int n, int form, int blocks, const MarchArgs& a, cudaStream_t s) {
   if (form == 3 && a.split_order == 2) {  // Strang: a half coupling before each propagation
+    if (n == 1024) return launch_one<1024, 2, 2, 3>(blocks, a, s);
     if (n == 2048) return launch_one<2048, 1, 2, 3>(blocks, a, s);
     if (n == 4096) return launch_one<4096, 1, 2, 3>(blocks, a, s);
     if (n == 8192) return launch_one<8192, 1, 2, 3>(blocks, a, s);

@@ -45,6 +45,12 @@ bool march_quad_use(int n, int split_order, int n_ch, int sms) {
   return each[i][o] * ((n_ch + sms - 1) / sms) < wave[i][o] * ((n_ch + per * sms - 1) / (per * sms));
 }
 
+size_t march_quad_smem_bytes(int n) {
+  return n == 256   ? Quad<256, 1>::smem_bytes()
+         : n == 512 ? Quad<512, 1>::smem_bytes()
+                    : Quad<1024, 1>::smem_bytes();
+}
+
 cudaError_t launch_march_quad(int n, const MarchArgs& a, cudaStream_t s) {
   if (n == 256) return launch_order<256>(a, s);
   if (n == 512) return launch_order<512>(a, s);

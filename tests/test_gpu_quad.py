@@ -63,3 +63,26 @@ def test_work_queue_singles_and_full_items_give_the_plans_bits(sms):
     b.close()
     for p in plans:
         p.close()
+
+
+@pytest.mark.parametrize("nx,order,n_ch", [(256, 1, 1700), (512, 2, 3), (1024, 1, 160),
+                                           (1024, 2, 310), (1024, 4, 307), (2048, 1, 5),
+                                           (2048, 4, 305), (4096, 1, 153), (4096, 4, 155),
+                                           (8192, 2, 3)])
+def test_default_forms_give_the_resident_forms_bits(nx, order, n_ch):
+    """A plan that names no form, on either side of the lines between forms."""
+    w = deformed_small(nx, nz=9, n_ch=n_ch, seed=nx + n_ch)
+    w.split_order = order
+    group = {256: 16, 512: 8, 1024: 4, 2048: 2}.get(nx, 1)
+    out = []
+    for forced in (False, True):
+        p = bpm.plan_from_workload(w)
+        if forced:
+            p.set_launch(form=0, channels_per_block=group)
+        p.run(4)
+        p.run(5)
+        p.sync()
+        out.append((p.e0(), p.eh(), *p.reflectivity()[:2]))
+        p.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
