@@ -59,6 +59,14 @@ BPM_DEV float2 c_fmas(float2 p, float s, float2 a) {
 #endif
   return make_float2(fmaf(p.x, s, a.x), fmaf(p.y, s, a.y));
 }
+// p * s per component
+BPM_DEV float2 c_scale(float2 p, float s) {
+#if BPM_PACKED_F32
+  return __fmul2_rn(p, make_float2(s, s));
+#else
+  return make_float2(p.x * s, p.y * s);
+#endif
+}
 BPM_DEV float2 c_mul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -240,6 +248,50 @@ BPM_DEV void dft4_bd(float2& a, float2& b, float2& c, float2& d) {
   a = c_fmas(P, BPM_C8, s0);
   c = c_fmas(P, -BPM_C8, s0);
   jout<INV, PJ>(d0, Q, BPM_C8, b, d);
+}
+
+// The same where each product is rounded by itself but one of two that meet in a
+// sum: d = W16^6 d is rounded, b's product fused (what the compiler makes of the
+// scalar separate form, FUSE = false and PA = false below).
+template <bool INV, bool PJ>
+BPM_DEV void dft4_bd_sep(float2& a, float2& b, float2& c, float2& d) {
+  const float2 pb = pre8<2, INV>(b), pd = pre8<6, INV>(d);
+  const float2 cd = c_scale(pd, BPM_C8), nd = c_scale(pd, -BPM_C8);
+  dft4_out<INV, PJ>(c_add(a, c), c_sub(a, c), c_fmas(pb, BPM_C8, cd), c_fmas(pb, BPM_C8, nd), a, b,
+                    c, d);
+}
+
+// 16-point DFT with the rounding of the scalar separate form (dft16_fwd / _inv
+// with FUSE = false, PA = false) in packed additions.
+template <bool INV, bool PJ = false>
+BPM_DEV void dft16_sep(float2 (&v)[16]) {
+  float2 o[16];
+  if constexpr (INV) {
+#pragma unroll
+    for (int m1 = 0; m1 < 4; ++m1)
+#pragma unroll
+      for (int m2 = 0; m2 < 4; ++m2) o[4 * m1 + m2] = v[m1 + 4 * m2];
+#pragma unroll
+    for (int m1 = 0; m1 < 4; ++m1) dft4<true, PJ>(o[4 * m1], o[4 * m1 + 1], o[4 * m1 + 2], o[4 * m1 + 3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) o[i] = v[i];
+#pragma unroll
+    for (int k2 = 0; k2 < 4; ++k2) dft4<false, PJ>(o[k2], o[k2 + 4], o[k2 + 8], o[k2 + 12]);
+  }
+  o[5] = w16<1, INV>(o[5]);
+  o[7] = w16<3, INV>(o[7]);
+  o[10] = w16<4, INV>(o[10]);
+  o[13] = w16<3, INV>(o[13]);
+  o[15] = w16<9, INV>(o[15]);
+  // rows 4 m1 + k2 (forward) or columns (inverse): index step 1 or 4 within a butterfly
+  constexpr int s = INV ? 4 : 1, r = INV ? 1 : 4;
+  dft4<INV, PJ>(o[0], o[s], o[2 * s], o[3 * s]);
+  dft4_c<2, INV, PJ>(o[r], o[r + s], o[r + 2 * s], o[r + 3 * s]);
+  dft4_bd_sep<INV, PJ>(o[2 * r], o[2 * r + s], o[2 * r + 2 * s], o[2 * r + 3 * s]);
+  dft4_c<6, INV, PJ>(o[3 * r], o[3 * r + s], o[3 * r + 2 * s], o[3 * r + 3 * s]);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[INV ? i : (i / 4) + 4 * (i % 4)] = o[i];
 }
 
 // 16-point DFT of v[0..15] as 4 x 4: k = 4 k1 + k2, m = m1 + 4 m2.
