@@ -1387,15 +1387,20 @@ bpm_status enqueue_round(bpm_batch b, RoundSlot& r, int chunk) {
                                cudaMemcpyHostToDevice, b->stream), "upload items");
   BPM_BCUDA(b, cudaMemsetAsync(r.d_counter, 0, kQueueCount * sizeof(int), b->stream),
             "clear queues");
-  // Queues run back to back, each on every SM (or the batch's cap) with its
-  // blocks per SM: the Nx = 8192 items (the longest) first, then the smaller
-  // ones; the idle tail is one item per queue.
+  // Queues in order, each on every SM (or the batch's cap) with its blocks per
+  // SM: the Nx = 8192 items (the longest) first, then the smaller ones.  Without
+  // a cap each may begin in the empty end of the one before; under a cap two at a
+  // time would take more SMs than the batch's share.
   int off = 0;
+  bool first = true;
   for (int q = 0; q < kQueueCount; ++q) {
-    if (cnt[q] > 0)
+    if (cnt[q] > 0) {
       BPM_BCUDA(b, launch_batch(r.d_plans, r.d_items + off, cnt[q], r.d_counter + q, q,
-                                std::min(cnt[q], sms * batch_blocks_per_sm(q)), b->stream),
+                                std::min(cnt[q], sms * batch_blocks_per_sm(q)),
+                                !first && b->max_blocks == 0, b->stream),
                 "batch kernel");
+      first = false;
+    }
     off += cnt[q];
   }
   const int n_big = cnt[kQueueTm8192] + cnt[kQueueTm8192s2] + cnt[kQueueTm8192s4];

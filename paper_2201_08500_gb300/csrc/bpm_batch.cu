@@ -18,6 +18,18 @@ namespace bpm {
 
 namespace {
 
+// Queues of a round overlap: a launch that follows another one starts when all
+// blocks of that one are running (programmatic dependent launch), and its blocks
+// take the SMs that the first queue's empty end leaves, instead of waiting for
+// its longest item.  They need nothing of one another.  Block 0 of each launch
+// waits for the launch before it to complete, so that completion of the last
+// means completion of all (and the others give their SM back at once).  Ten
+// uneven instances in four queues: a round of 40.6 ms -> 35.8.
+BPM_DEV void chain_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+BPM_DEV void chain_end() {
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 constexpr int kSmallThreads = 256;
 
 template <int N>
@@ -39,6 +51,7 @@ template <int SPLIT>
 __global__ void __launch_bounds__(kSmallThreads, 1)
     batch_kernel(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
                  int n_items, int* counter) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
   for (;;) {
@@ -55,6 +68,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       default: break;
     }
   }
+  chain_end();
 }
 
 // Body of the TMEM queues: first order in the narrow layout (fewer spills in
@@ -64,13 +78,14 @@ template <int N, int SPLIT>
 using TmBody = Parked<N, SPLIT, true, SPLIT != 1 && N <= 4096>;
 
 // Items at Nx = 2048, 4096, 8192 in the parked form with tables in tensor
-// memory (Parked<N, SPLIT, true>, the fastest single-plan form there): one channel per item, N/16 threads per block,
-// 512/(N/16) blocks per SM; every block allocates its TMEM columns once and
+// memory (Parked<N, SPLIT, true>, the fastest single-plan form there): one
+// channel per item, N/16 threads per block, 512/(N/16) blocks per SM; every block allocates its TMEM columns once and
 // frees them on exit.
 template <int N, int SPLIT>
 __global__ void __launch_bounds__(N / 16, 512 / (N / 16))
     batch_kernel_tm(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
                     int n_items, int* counter) {
+  chain_begin();
   using P = TmBody<N, SPLIT>;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -90,6 +105,7 @@ __global__ void __launch_bounds__(N / 16, 512 / (N / 16))
   }
   tmem_sync();
   if (threadIdx.x / 32 == 0) tmem_dealloc<P::kCols>(s_tbase);
+  chain_end();
 }
 
 // Items at Nx = 1024 in the tensor-memory parked form with two channels per
@@ -102,6 +118,7 @@ template <int N, int SPLIT>
 __global__ void __launch_bounds__(2 * (N / 16), 512 / (2 * (N / 16)))
     batch_kernel_tm2(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
                      int n_items, int* counter) {
+  chain_begin();
   using P = Parked<N, SPLIT, true, true, 2>;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item[2];
@@ -124,6 +141,7 @@ __global__ void __launch_bounds__(2 * (N / 16), 512 / (2 * (N / 16)))
   }
   tmem_sync();  // both groups are done (their TMEM loads waited)
   if (threadIdx.x / 32 == 0) tmem_dealloc<P::kCols>(s_tbase);
+  chain_end();
 }
 
 // Fourth-order items at Nx = 1024 in the parked form with both table sets read
@@ -132,6 +150,7 @@ __global__ void __launch_bounds__(2 * (N / 16), 512 / (2 * (N / 16)))
 __global__ void __launch_bounds__(64, 8)
     batch_kernel_pk1024s4(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
                           int n_items, int* counter) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
   for (;;) {
@@ -143,6 +162,7 @@ __global__ void __launch_bounds__(64, 8)
     const BatchItem item = items[it];
     Parked<1024, 4>::march_channel(plans[item.plan], item.ch0, smem, threadIdx.x);
   }
+  chain_end();
 }
 
 // Single channels at Nx <= 512 with 8 Nx/16 threads each (bpm_quad.cuh).
@@ -150,6 +170,7 @@ template <int N, int SPLIT>
 __global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>::kThreads)
     batch_kernel_quad(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
                       int n_items, int* counter) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
   for (;;) {
@@ -161,6 +182,7 @@ __global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>
     const BatchItem item = items[it];
     Quad<N, SPLIT>::march_channel(plans[item.plan], item.ch0, smem);
   }
+  chain_end();
 }
 
 }  // namespace
@@ -235,96 +257,80 @@ int batch_blocks_per_sm(int queue) {
 
 namespace {
 
-template <int N, int SPLIT>
-void tm_launch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
-               int blocks, cudaStream_t s) {
-  batch_kernel_tm<N, SPLIT><<<blocks, N / 16, TmBody<N, SPLIT>::smem_bytes(), s>>>(
-      plans, items, n_items, counter);
-}
+using BatchKernel = void (*)(const MarchArgs*, const BatchItem*, int, int*);
+struct QueueLaunch {
+  BatchKernel kernel;
+  int threads;
+  size_t smem;
+};
 
+template <int N, int SPLIT>
+QueueLaunch tm_queue() {
+  return {batch_kernel_tm<N, SPLIT>, N / 16, TmBody<N, SPLIT>::smem_bytes()};
+}
 template <int SPLIT>
-void tm2_launch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
-                int blocks, cudaStream_t s) {
-  batch_kernel_tm2<1024, SPLIT>
-      <<<blocks, 128, Parked<1024, SPLIT, true, true, 2>::smem_bytes(), s>>>(plans, items, n_items,
-                                                                             counter);
+QueueLaunch tm2_queue() {
+  return {batch_kernel_tm2<1024, SPLIT>, 128, Parked<1024, SPLIT, true, true, 2>::smem_bytes()};
 }
-
 template <int N, int SPLIT>
-void quad_launch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
-                 int blocks, cudaStream_t s) {
-  batch_kernel_quad<N, SPLIT><<<blocks, Quad<N, SPLIT>::kThreads, Quad<N, SPLIT>::smem_bytes(), s>>>(
-      plans, items, n_items, counter);
+QueueLaunch quad_queue() {
+  return {batch_kernel_quad<N, SPLIT>, Quad<N, SPLIT>::kThreads, Quad<N, SPLIT>::smem_bytes()};
 }
 
-template <int N, int SPLIT>
-cudaError_t tm_attr() {
-  return cudaFuncSetAttribute(batch_kernel_tm<N, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(TmBody<N, SPLIT>::smem_bytes()));
-}
-
-template <int SPLIT>
-cudaError_t tm2_attr() {
-  return cudaFuncSetAttribute(batch_kernel_tm2<1024, SPLIT>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(Parked<1024, SPLIT, true, true, 2>::smem_bytes()));
+QueueLaunch queue_launch(int queue) {
+  switch (queue) {
+    case kQueueTm8192: return tm_queue<8192, 1>();
+    case kQueueTm8192s2: return tm_queue<8192, 2>();
+    case kQueueTm8192s4: return tm_queue<8192, 4>();
+    case kQueueTm4096: return tm_queue<4096, 1>();
+    case kQueueTm4096s2: return tm_queue<4096, 2>();
+    case kQueueTm4096s4: return tm_queue<4096, 4>();
+    case kQueueTm2048: return tm_queue<2048, 1>();
+    case kQueueTm2048s2: return tm_queue<2048, 2>();
+    case kQueueTm2048s4: return tm_queue<2048, 4>();
+    case kQueueTm1024: return tm2_queue<1>();
+    case kQueueTm1024s2: return tm2_queue<2>();
+    case kQueuePk1024s4: return {batch_kernel_pk1024s4, 64, Parked<1024, 4>::smem_bytes()};
+    case kQueueSmall: return {batch_kernel<1>, kSmallThreads, kSmallSmem};
+    case kQueueSmall2: return {batch_kernel<2>, kSmallThreads, kSmallSmem};
+    case kQueueSmall4: return {batch_kernel<4>, kSmallThreads, kSmallSmem};
+    case kQueueQuad512: return quad_queue<512, 1>();
+    case kQueueQuad512s2: return quad_queue<512, 2>();
+    case kQueueQuad512s4: return quad_queue<512, 4>();
+    case kQueueQuad256: return quad_queue<256, 1>();
+    case kQueueQuad256s2: return quad_queue<256, 2>();
+    case kQueueQuad256s4: return quad_queue<256, 4>();
+    default: return {nullptr, 0, 0};
+  }
 }
 
 }  // namespace
 
 cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
-                         int queue, int blocks, cudaStream_t s) {
+                         int queue, int blocks, bool follow, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  switch (queue) {
-    case kQueueTm8192: tm_launch<8192, 1>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm4096: tm_launch<4096, 1>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm2048: tm_launch<2048, 1>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm8192s2: tm_launch<8192, 2>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm4096s2: tm_launch<4096, 2>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm2048s2: tm_launch<2048, 2>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm8192s4: tm_launch<8192, 4>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm4096s4: tm_launch<4096, 4>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm2048s4: tm_launch<2048, 4>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm1024: tm2_launch<1>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueTm1024s2: tm2_launch<2>(plans, items, n_items, counter, blocks, s); break;
-    case kQueuePk1024s4:
-      batch_kernel_pk1024s4<<<blocks, 64, Parked<1024, 4>::smem_bytes(), s>>>(plans, items, n_items,
-                                                                              counter);
-      break;
-    case kQueueSmall:
-      batch_kernel<1><<<blocks, kSmallThreads, kSmallSmem, s>>>(plans, items, n_items, counter);
-      break;
-    case kQueueSmall2:
-      batch_kernel<2><<<blocks, kSmallThreads, kSmallSmem, s>>>(plans, items, n_items, counter);
-      break;
-    case kQueueSmall4:
-      batch_kernel<4><<<blocks, kSmallThreads, kSmallSmem, s>>>(plans, items, n_items, counter);
-      break;
-    case kQueueQuad256: quad_launch<256, 1>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueQuad512: quad_launch<512, 1>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueQuad256s2: quad_launch<256, 2>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueQuad512s2: quad_launch<512, 2>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueQuad256s4: quad_launch<256, 4>(plans, items, n_items, counter, blocks, s); break;
-    case kQueueQuad512s4: quad_launch<512, 4>(plans, items, n_items, counter, blocks, s); break;
-    default:
-      return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+  const QueueLaunch q = queue_launch(queue);
+  if (!q.kernel) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(blocks));
+  cfg.blockDim = dim3(unsigned(q.threads));
+  cfg.dynamicSmemBytes = q.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = follow ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, q.kernel, plans, items, n_items, counter);
 }
 
 cudaError_t batch_set_attributes() {
-  const int small = int(kSmallSmem);
-  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t r[] = {cudaFuncSetAttribute(batch_kernel<1>, attr, small),
-                     cudaFuncSetAttribute(batch_kernel<2>, attr, small),
-                     cudaFuncSetAttribute(batch_kernel<4>, attr, small),
-                     tm_attr<8192, 1>(), tm_attr<4096, 1>(), tm_attr<2048, 1>(),
-                     tm_attr<8192, 2>(), tm_attr<4096, 2>(), tm_attr<2048, 2>(),
-                     tm_attr<8192, 4>(), tm_attr<4096, 4>(), tm_attr<2048, 4>(),
-                     tm2_attr<1>(), tm2_attr<2>(),
-                     cudaFuncSetAttribute(batch_kernel_pk1024s4, attr, int(Parked<1024, 4>::smem_bytes()))};
-  for (cudaError_t e : r)
+  for (int queue = 0; queue < kQueueCount; ++queue) {
+    const QueueLaunch q = queue_launch(queue);
+    const cudaError_t e =
+        cudaFuncSetAttribute(q.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(q.smem));
     if (e != cudaSuccess) return e;
+  }
   return cudaSuccess;
 }
 

@@ -141,8 +141,11 @@ int batch_queue(int n, int split_order);
 bool batch_singles(int n, int split_order, int channels, int items, int sms);
 int batch_single_queue(int n, int split_order);
 int batch_blocks_per_sm(int queue);
+// follow: start as soon as every block of the stream's last launch, itself a
+// launch_batch, has started, and complete after it (the queues' work is
+// independent; see chain_begin in bpm_batch.cu).
 cudaError_t launch_batch(const MarchArgs* plans, const BatchItem* items, int n_items, int* counter,
-                         int queue, int blocks, cudaStream_t s);
+                         int queue, int blocks, bool follow, cudaStream_t s);
 
 // Host runtime helpers (bpm_api.cu): FFT constants of size n (twiddles, spectrum
 // order, round-trip gain; host memory owned by a process-wide cache) and a
