@@ -257,7 +257,7 @@ struct bpm_plan_s {
   double* trans = nullptr;
   double2* eh_time = nullptr;
   double2* time_tab = nullptr;   // tables of the frequency-to-time transform (null: direct sum)
-  int* dflag = nullptr;
+  int* dflag = nullptr;          // [0] no Bragg solution, [1] bulk-copy wait, from kHandoff: march_shares
   NormScratch* norm_scratch = nullptr;
   double* u_tmp = nullptr;
   float* gcorr = nullptr;        // 3D: curvature factor per column
@@ -385,6 +385,8 @@ void apply_launch(bpm_plan p, int form, int group) {
                                         : march_smem_bytes(nx, group));
 }
 
+constexpr size_t kHandoff = 4;  // first of the shares' marks in dflag
+
 size_t plan_bytes(const bpm_grid& g, int n_ch) {
   const size_t plane = size_t(g.nx) * (g.dims == 3 ? g.ny : 1);
   const size_t nf = size_t(n_ch) * plane;
@@ -500,7 +502,8 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
   check(dalloc(&p->trans, size_t(n_channels)), "alloc T");
   check(dalloc(&p->eh_time, nf), "alloc time response");
   check(dalloc(&p->time_tab, time_table_elems(n_channels)), "alloc time tables");
-  check(dalloc(&p->dflag, size_t(4)), "alloc status");
+  const size_t n_flags = kHandoff + size_t(kSharesPerSm) * device_info().sm_count;
+  check(dalloc(&p->dflag, n_flags), "alloc status");
   check(dalloc(&p->norm_scratch, size_t(1)), "alloc norm parts");
   if (g.dims == 3) {
     check(dalloc(&p->gcorr, size_t(n_channels) * 2 * g.nx), "alloc curvature factors");
@@ -536,7 +539,7 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
   check(cudaMemcpyAsync(p->gain, fc.gain.data(), sizeof(double) * g.nx, cudaMemcpyHostToDevice,
                         p->stream),
         "upload gain");
-  check(cudaMemsetAsync(p->dflag, 0, sizeof(int) * 4, p->stream), "clear status");
+  check(cudaMemsetAsync(p->dflag, 0, sizeof(int) * n_flags, p->stream), "clear status");
   check(cudaMemsetAsync(p->norm_scratch, 0, sizeof(NormScratch), p->stream), "clear norm parts");
   check(launch_time_tables(n_channels, p->time_tab, p->stream), "time tables");
   std::vector<float2> qyt;
@@ -816,6 +819,10 @@ BPM_API bpm_status bpm_run(bpm_plan p, int n_steps) {
     if (!p->chosen)
       march_default_form(p->grid.nx, a.split_order, p->n_ch, device_info().sm_count, &form, &group);
     apply_launch(p, form, group);
+    const int sms = device_info().sm_count;
+    a.per_sm = march_shares(p->grid.nx, a.split_order, form, group, p->n_ch, n_steps, sms);
+    a.handoff = p->dflag + kHandoff;
+    if (a.per_sm) p->stats.blocks = p->blocks = a.per_sm * sms;
     if (form == 1 && a.split_order == 1)
       BPM_CUDA(p, launch_march_l2(p->grid.nx, group, p->blocks, a, p->stream), "march kernel");
     else if ((form == 2 && a.split_order != 2) || (form == 3 && a.split_order <= 2))

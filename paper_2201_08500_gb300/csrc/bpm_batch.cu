@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(N / 16, 512 / (N / 16))
     if (it >= n_items) break;
     const BatchItem item = items[it];
     const MarchArgs& A = plans[item.plan];
-    if (item.ch0 < A.n_ch) P::march_channel(A, item.ch0, smem, threadIdx.x, tcol);
+    if (item.ch0 < A.n_ch) P::march_channel(A, item.ch0, A.z0, A.n_steps, smem, threadIdx.x, tcol);
   }
   tmem_sync();
   if (threadIdx.x / 32 == 0) tmem_dealloc<P::kCols>(s_tbase);
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(2 * (N / 16), 512 / (2 * (N / 16)))
     if (it >= n_items) break;
     const BatchItem item = items[it];
     const MarchArgs& A = plans[item.plan];
-    if (item.ch0 < A.n_ch) P::march_channel(A, item.ch0, gsmem, t, tcol);
+    if (item.ch0 < A.n_ch) P::march_channel(A, item.ch0, A.z0, A.n_steps, gsmem, t, tcol);
   }
   tmem_sync();  // both groups are done (their TMEM loads waited)
   if (threadIdx.x / 32 == 0) tmem_dealloc<P::kCols>(s_tbase);
@@ -160,7 +160,8 @@ __global__ void __launch_bounds__(64, 8)
     const int it = s_item;
     if (it >= n_items) break;
     const BatchItem item = items[it];
-    Parked<1024, 4>::march_channel(plans[item.plan], item.ch0, smem, threadIdx.x);
+    const MarchArgs& A = plans[item.plan];
+    Parked<1024, 4>::march_channel(A, item.ch0, A.z0, A.n_steps, smem, threadIdx.x);
   }
   chain_end();
 }
@@ -180,7 +181,8 @@ __global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>
     const int it = s_item;
     if (it >= n_items) break;
     const BatchItem item = items[it];
-    Quad<N, SPLIT>::march_channel(plans[item.plan], item.ch0, smem);
+    const MarchArgs& A = plans[item.plan];
+    Quad<N, SPLIT>::march_channel(A, item.ch0, A.z0, A.n_steps, smem);
   }
   chain_end();
 }

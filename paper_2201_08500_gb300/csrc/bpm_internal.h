@@ -70,6 +70,8 @@ struct MarchArgs {
   int z0;
   int n_steps;
   int split_order;           // Eq. split-op: 1, 2 (Strang) or 4 (tables and coef then hold two sets)
+  int per_sm = 0;            // > 0: equal shares for this many blocks an SM (bpm_share.cuh)
+  int* handoff = nullptr;    // a zero a slot, left as it was found
 };
 
 // Arguments of the 3D row / column passes (bpm_3d.cu).
@@ -170,7 +172,13 @@ cudaError_t launch_march_strang(int n, int group, int blocks, const MarchArgs& a
 // order: launch_march takes it for one channel a block where it is the faster.
 bool march_quad_use(int n, int split_order, int n_ch, int sms);
 size_t march_quad_smem_bytes(int n);
-cudaError_t launch_march_quad(int n, const MarchArgs& a, cudaStream_t s);
+cudaError_t launch_march_quad(int n, int blocks, const MarchArgs& a, cudaStream_t s);
+cudaError_t march_set_attributes_quad();
+// Blocks an SM of a march in equal shares (bpm_share.cuh), 0 for one channel a
+// group in turn.
+int march_shares(int n, int split_order, int form, int group, int n_ch, int n_steps, int sms);
+// Marks a plan keeps for it: one a slot.
+constexpr int kSharesPerSm = 8;
 // Second form of the first-order march: propagator tables and stage twiddles
 // read from L2 instead of shared memory / registers, at most 128 registers, so
 // that two blocks (two channel groups at independent FFT phases) share an SM.

@@ -17,6 +17,9 @@
 // reflectivity / transmissivity sums are reduced in FP64.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "bpm_march_impl.cuh"
 
 namespace bpm {
@@ -80,6 +83,70 @@ void march_default_form(int n, int split_order, int n_ch, int sms, int* form, in
   }
 }
 
+namespace {
+
+// us a step with k = 1, 2, ... blocks on every SM (as many as fit), 152 SMs.
+struct StepTimes {
+  int n, form, order;  // form 0: bpm_quad.cuh
+  float t[8];
+};
+constexpr StepTimes kStepTimes[] = {
+    {256, 0, 1, {0.63f, 0.75f, 0.84f, 1.04f, 1.26f, 1.49f}},
+    {256, 0, 2, {0.92f, 1.02f, 1.10f, 1.26f, 1.46f, 1.64f}},
+    {256, 0, 4, {2.67f, 3.00f, 3.30f, 3.95f, 4.62f, 5.65f}},
+    {512, 0, 1, {1.05f, 1.44f, 1.95f}},
+    {512, 0, 2, {1.26f, 1.54f, 2.07f}},
+    {512, 0, 4, {3.77f, 5.12f, 7.32f}},
+    {1024, 0, 1, {1.79f}},
+    {1024, 0, 2, {1.97f}},
+    {1024, 0, 4, {5.40f}},
+    {1024, 2, 1, {2.86f, 3.15f, 4.53f, 4.85f, 5.95f, 6.45f, 7.82f, 8.23f}},
+    {1024, 2, 4, {9.46f, 12.1f, 14.8f, 15.7f, 18.9f, 20.2f, 24.2f, 25.4f}},
+    {1024, 3, 1, {3.06f, 4.24f, 5.74f, 7.35f}},
+    {1024, 3, 2, {3.92f, 4.83f, 6.40f, 8.29f}},
+    {2048, 2, 1, {4.12f, 5.30f, 6.85f, 8.71f}},
+    {2048, 2, 4, {13.8f, 16.0f, 21.7f, 27.4f}},
+    {2048, 3, 1, {4.11f, 4.46f, 6.18f, 7.97f}},
+    {2048, 3, 2, {4.91f, 5.14f, 7.13f, 8.91f}},
+    {4096, 2, 1, {6.65f, 9.78f}},
+    {4096, 2, 4, {18.2f, 28.7f}},
+    {4096, 3, 1, {5.27f, 8.72f}},
+    {4096, 3, 2, {6.04f, 9.33f}},
+    {8192, 0, 1, {10.5f}},
+    {8192, 0, 2, {11.6f}},
+    {8192, 0, 4, {34.5f}},
+};
+
+}  // namespace
+
+// With r blocks' worth of channels an SM, the launch of whole channels takes the
+// time of ceil(r) blocks on an SM while they fit and ceil(r) / kmax that of the
+// kmax that do beyond; equal shares on k <= r blocks an SM take r / k of theirs.
+// E.g. (us a step, whole channels -> shares) 512 channels of 8192 points
+// 41.3 -> 35.6; 400 of 4096 13.0 -> 11.5; 700 of 2048 10.1 -> 9.1; 611 of 1024
+// 5.7 -> 4.3, 1024 of 1024 7.3 -> 6.4 with three blocks an SM.
+// Beyond kmax blocks that end at different times fill some of the gap by
+// themselves where several share an SM (1024 of 4096: 29.0, in shares 29.3): 5 %
+// has to be expected there.  A share's extra piece costs about a step, so short
+// runs take whole channels.
+int march_shares(int n, int split_order, int form, int group, int n_ch, int n_steps, int sms) {
+  if (n == 8192) form = 0;
+  if (n_steps < 16 || sms < 1 || form == 1) return 0;
+  if (form == 0 && n != 8192 && (group != 1 || !march_quad_use(n, split_order, n_ch, sms))) return 0;
+  const StepTimes* s = nullptr;
+  for (const StepTimes& row : kStepTimes)
+    if (row.n == n && row.form == form && row.order == split_order) s = &row;
+  if (!s) return 0;
+  int kmax = 1;
+  while (kmax < 8 && s->t[kmax] > 0.f) ++kmax;
+  const double r = double((n_ch + group - 1) / group) / sms;
+  const int up = int(std::ceil(r)), k = std::min(int(r), kmax);
+  if (k < 1 || k * sms * group >= n_ch) return 0;
+  const double whole = up <= kmax ? s->t[up - 1] : double(up) / kmax * s->t[kmax - 1];
+  const double shared = double(n_ch) / (group * sms) / k * s->t[k - 1];
+  return whole > (up > kmax && kmax > 1 ? 1.05 : 1.015) * shared ? k : 0;
+}
+
 size_t march_smem_bytes(int n, int group) {
 #define BPM_SMEM_CASE(NN, GG) \
   if (n == NN && group == GG) return MarchBody<NN, GG, 1, 0>::type::smem_bytes();
@@ -95,6 +162,7 @@ size_t march_smem_bytes(int n, int group) {
 cudaError_t march_set_attributes() {
   cudaError_t e = march_set_attributes_strang();
   if (cudaError_t e4 = march_set_attributes_split4(); e4 != cudaSuccess) e = e4;
+  if (cudaError_t eq = march_set_attributes_quad(); eq != cudaSuccess) e = eq;
   cudaError_t r[] = {attr_one<256, 1, 1>(),  attr_one<256, 16, 1>(),
                      attr_one<512, 1, 1>(),  attr_one<512, 8, 1>(),
                      attr_one<1024, 1, 1>(), attr_one<1024, 4, 1>(),
@@ -108,7 +176,7 @@ cudaError_t march_set_attributes() {
 cudaError_t launch_march(int n, int group, int blocks, const MarchArgs& a, cudaStream_t s) {
   int sms = 0;
   if (group == 1 && device_ready(&sms) && march_quad_use(n, a.split_order, a.n_ch, sms))
-    return launch_march_quad(n, a, s);
+    return launch_march_quad(n, blocks, a, s);
   if (a.split_order == 2) return launch_march_strang(n, group, blocks, a, s);
   if (a.split_order == 4) return launch_march_split4(n, group, blocks, a, s);
 #define BPM_LAUNCH_CASE(NN, GG) \

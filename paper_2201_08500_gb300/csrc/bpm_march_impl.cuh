@@ -59,7 +59,8 @@ __global__ void __launch_bounds__((N / 16) * G, march_min_blocks(N, G, FORM))
 template <int N, int G, int SPLIT, int FORM = 0>
 cudaError_t launch_one(int blocks, const MarchArgs& a, cudaStream_t s) {
   march_kernel<N, G, SPLIT, FORM>
-      <<<blocks, (N / 16) * G, MarchBody<N, G, SPLIT, FORM>::type::smem_bytes(), s>>>(a);
+      <<<blocks, (N / 16) * G, share_smem(MarchBody<N, G, SPLIT, FORM>::type::smem_bytes(), a.per_sm),
+         s>>>(a);
   return cudaGetLastError();
 }
 
@@ -67,7 +68,7 @@ template <int N, int G, int SPLIT, int FORM = 0>
 cudaError_t attr_one() {
   return cudaFuncSetAttribute(march_kernel<N, G, SPLIT, FORM>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(MarchBody<N, G, SPLIT, FORM>::type::smem_bytes()));
+                              int(share_smem(MarchBody<N, G, SPLIT, FORM>::type::smem_bytes(), 1)));
 }
 
 }  // namespace

@@ -15,17 +15,17 @@ __global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>
 }
 
 template <int N, int SPLIT>
-cudaError_t launch_one(const MarchArgs& a, cudaStream_t s) {
-  march_quad_kernel<N, SPLIT>
-      <<<a.n_ch, Quad<N, SPLIT>::kThreads, Quad<N, SPLIT>::smem_bytes(), s>>>(a);
+cudaError_t launch_one(int blocks, const MarchArgs& a, cudaStream_t s) {
+  march_quad_kernel<N, SPLIT><<<blocks, Quad<N, SPLIT>::kThreads,
+                                share_smem(Quad<N, SPLIT>::smem_bytes(), a.per_sm), s>>>(a);
   return cudaGetLastError();
 }
 
 template <int N>
-cudaError_t launch_order(const MarchArgs& a, cudaStream_t s) {
-  if (a.split_order == 2) return launch_one<N, 2>(a, s);
-  if (a.split_order == 4) return launch_one<N, 4>(a, s);
-  return launch_one<N, 1>(a, s);
+cudaError_t launch_order(int blocks, const MarchArgs& a, cudaStream_t s) {
+  if (a.split_order == 2) return launch_one<N, 2>(blocks, a, s);
+  if (a.split_order == 4) return launch_one<N, 4>(blocks, a, s);
+  return launch_one<N, 1>(blocks, a, s);
 }
 
 }  // namespace
@@ -51,11 +51,29 @@ size_t march_quad_smem_bytes(int n) {
                     : Quad<1024, 1>::smem_bytes();
 }
 
-cudaError_t launch_march_quad(int n, const MarchArgs& a, cudaStream_t s) {
-  if (n == 256) return launch_order<256>(a, s);
-  if (n == 512) return launch_order<512>(a, s);
-  if (n == 1024) return launch_order<1024>(a, s);
+cudaError_t launch_march_quad(int n, int blocks, const MarchArgs& a, cudaStream_t s) {
+  if (n == 256) return launch_order<256>(blocks, a, s);
+  if (n == 512) return launch_order<512>(blocks, a, s);
+  if (n == 1024) return launch_order<1024>(blocks, a, s);
   return cudaErrorInvalidValue;
+}
+
+namespace {
+template <int N, int SPLIT>
+cudaError_t attr_one() {
+  return cudaFuncSetAttribute(march_quad_kernel<N, SPLIT>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              int(share_smem(Quad<N, SPLIT>::smem_bytes(), 1)));
+}
+}  // namespace
+
+cudaError_t march_set_attributes_quad() {
+  cudaError_t r[] = {attr_one<256, 1>(), attr_one<256, 2>(),  attr_one<256, 4>(),
+                     attr_one<512, 1>(), attr_one<512, 2>(),  attr_one<512, 4>(),
+                     attr_one<1024, 1>(), attr_one<1024, 2>(), attr_one<1024, 4>()};
+  for (cudaError_t e : r)
+    if (e != cudaSuccess) return e;
+  return cudaSuccess;
 }
 
 }  // namespace bpm

@@ -46,7 +46,9 @@
 
 #include <cuda_runtime.h>
 
+#include "bpm_norm.cuh"
 #include "bpm_resident.cuh"
+#include "bpm_share.cuh"
 #include "bpm_tmem.cuh"
 
 namespace bpm {
@@ -431,18 +433,20 @@ struct Parked {
 #pragma unroll
     for (int e = 0; e < 2; ++e)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        float4 tv[4];
+      for (int h = 0; h < 2; ++h) {
+        float4 tv[2][4];  // eight loads in flight
 #pragma unroll
-        for (int i = 0; i < 4; ++i) tv[i] = __ldg(gtab + e * N + (4 * c + i) * T + t);
-        tmem_st16(tcol + uint32_t(64 * e + 16 * c), tv);
+        for (int i = 0; i < 8; ++i) tv[i / 4][i % 4] = __ldg(gtab + e * N + (8 * h + i) * T + t);
+        tmem_st16(tcol + uint32_t(64 * e + 32 * h), tv[0]);
+        tmem_st16(tcol + uint32_t(64 * e + 32 * h + 16), tv[1]);
       }
     tmem_wait_st();
   }
 
-  // March channel ch of plan A by A.n_steps steps (this block: T threads).
-  static BPM_DEV void march_channel(const MarchArgs& A, int ch, unsigned char* smem, int t,
-                                    uint32_t tcol = 0) {
+  // March channel ch of plan A by n steps from row z0 (this block: T threads).
+  // open: nonzero if the sums of |E|^2 are not needed, being those of a part.
+  static BPM_DEV void march_channel(const MarchArgs& A, int ch, int z0, int n, unsigned char* smem,
+                                    int t, uint32_t tcol = 0, const int* open = nullptr) {
     float2* x = reinterpret_cast<float2*>(smem);
     double* red = reinterpret_cast<double*>(park_of(x, 2));
     const float4* gtab = A.tables + size_t(ch) * kTabs * 2 * N;
@@ -451,9 +455,11 @@ struct Parked {
     // so is the crystal's extent (see couple)
     ChannelCoef* scf = reinterpret_cast<ChannelCoef*>(red + 32);
     unsigned* mask = reinterpret_cast<unsigned*>(red + 40);
+    int* z_end = reinterpret_cast<int*>(red + 41);
     if (SPLIT == 1 && t == 0) scf[0] = A.coef[ch];
     if (t == 0) {
       const int lo = __ldg(A.ext), hi = -__ldg(A.ext + 1);  // crystal cells [lo, hi)
+      *z_end = z0 + n;
       *mask = lo == kExtNone ? 0u : (2u << ((hi - 1) / T)) - (1u << (lo / T));
     }
     gsync();
@@ -470,8 +476,8 @@ struct Parked {
     park(v, park_of(x, 1), t);
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = e0[t + T * k];
-    for (int step = 0; step < A.n_steps; ++step) {
-      const float2* crow = A.cfield + size_t(A.z0 + step) * N;
+    for (int z = z0; z < *z_end; ++z) {
+      const float2* crow = A.cfield + size_t(z) * N;
       if constexpr (SPLIT == 4) {
         const ChannelCoef cf1 = A.coef[size_t(ch) * 2 + 1];
         couple(v, park_of(x, held ^ 1), held, crow, cf, mask, t);
@@ -489,13 +495,19 @@ struct Parked {
     // sums of |E|^2 of the envelope in v and of the parked one
     float2 *fv = held ? eh : e0, *fp = held ? e0 : eh;
     double sv = 0.0, sp = 0.0;
+    const bool sums = !open || !*open;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       const float2 m = parked(park_of(x, held ^ 1), t, k);
       fv[t + T * k] = v[k];
       fp[t + T * k] = m;
-      sv += double(v[k].x) * v[k].x + double(v[k].y) * v[k].y;
-      sp += double(m.x) * m.x + double(m.y) * m.y;
+      if (!sums) continue;
+      sv = add_norm(sv, v[k]);
+      sp = add_norm(sp, m);
+    }
+    if (!sums) {
+      gsync();
+      return;
     }
     double sa = held ? sp : sv, sb = held ? sv : sp;
 #pragma unroll
@@ -528,18 +540,25 @@ struct Parked {
     const int grp = G == 1 ? 0 : tid / T;  // channel group of this thread
     const int t = G == 1 ? tid : tid % T;
     unsigned char* gsmem = G == 1 ? smem : smem + size_t(grp) * group_bytes();
+    __shared__ uint32_t s_tbase;
+    __shared__ Share s_share[G];
     if constexpr (TMEM) {
-      __shared__ uint32_t s_tbase;
       if (tid / 32 == 0) tmem_alloc<kCols>(&s_tbase);
       tmem_sync();
-      const uint32_t tbase = s_tbase;
-      for (int ch = blockIdx.x * G + grp; ch < A.n_ch; ch += gridDim.x * G)
-        march_channel(A, ch, gsmem, t, tmem_thread(tbase, tid));
+    }
+    const uint32_t tcol = TMEM ? tmem_thread(s_tbase, tid) : 0;
+    const int slot = blockIdx.x * G + grp, slots = gridDim.x * G;
+    Share* share = &s_share[grp];
+    if (t == 0) share_begin(A, slot, slots, share);
+    for (;;) {
+      if (t == 0) share_next(A, slot, slots, share);
+      gsync();
+      if (share->ch < 0) break;
+      march_channel(A, share->ch, share->z0, share->n, gsmem, t, tcol, &share->open);
+    }
+    if constexpr (TMEM) {
       tmem_sync();  // every thread's TMEM loads have completed (waited)
-      if (tid / 32 == 0) tmem_dealloc<kCols>(tbase);
-    } else {
-      for (int ch = blockIdx.x * G + grp; ch < A.n_ch; ch += gridDim.x * G)
-        march_channel(A, ch, gsmem, t);
+      if (tid / 32 == 0) tmem_dealloc<kCols>(s_tbase);
     }
   }
 };

@@ -23,7 +23,9 @@
 
 #include <cuda_runtime.h>
 
+#include "bpm_norm.cuh"
 #include "bpm_resident.cuh"
+#include "bpm_share.cuh"
 
 namespace bpm {
 
@@ -206,8 +208,8 @@ struct Quad {
     }
   }
 
-  // March channel ch of plan A (this block: kThreads threads).
-  static BPM_DEV void march_channel(const MarchArgs& A, int ch, unsigned char* smem) {
+  // March channel ch of plan A by n steps from row z0 (this block: kThreads threads).
+  static BPM_DEV void march_channel(const MarchArgs& A, int ch, int z0, int n, unsigned char* smem) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     Ctx c;
     c.env = lane >> 4;
@@ -234,8 +236,8 @@ struct Quad {
     float2 v[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = field[t + T * (q + 4 * i)];
-    const float2* crow = A.cfield + size_t(A.z0) * N + t + T * q;
-    for (int step = 0; step < A.n_steps; ++step, crow += N) {
+    const float2* crow = A.cfield + size_t(z0) * N + t + T * q;
+    for (int step = 0; step < n; ++step, crow += N) {
       float2 cc[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) cc[i] = __ldg(crow + 4 * T * i);
@@ -268,7 +270,7 @@ struct Quad {
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         const float2 f = buf[e * kSlots + tt + T * k];
-        s += double(f.x) * f.x + double(f.y) * f.y;
+        s = add_norm(s, f);
       }
       constexpr int W = T < 32 ? T : 32;
 #pragma unroll
@@ -292,7 +294,14 @@ struct Quad {
   }
 
   static BPM_DEV void run(const MarchArgs& A, unsigned char* smem) {
-    for (int ch = blockIdx.x; ch < A.n_ch; ch += gridDim.x) march_channel(A, ch, smem);
+    __shared__ Share share;
+    if (threadIdx.x == 0) share_begin(A, blockIdx.x, gridDim.x, &share);
+    for (;;) {
+      if (threadIdx.x == 0) share_next(A, blockIdx.x, gridDim.x, &share);
+      __syncthreads();
+      if (share.ch < 0) break;
+      march_channel(A, share.ch, share.z0, share.n, smem);
+    }
   }
 };
 

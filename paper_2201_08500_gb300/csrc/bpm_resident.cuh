@@ -6,6 +6,7 @@
 
 #include "bpm_fft.cuh"
 #include "bpm_internal.h"
+#include "bpm_norm.cuh"
 
 namespace bpm {
 
@@ -318,8 +319,8 @@ struct Resident {
     for (int k = 0; k < 16; ++k) {
       e0[t + T * k] = a[k];
       eh[t + T * k] = b[k];
-      sa += double(a[k].x) * a[k].x + double(a[k].y) * a[k].y;
-      sb += double(b[k].x) * b[k].x + double(b[k].y) * b[k].y;
+      sa = add_norm(sa, a[k]);
+      sb = add_norm(sb, b[k]);
     }
     // reduce over the T threads of this channel
     constexpr int W = T < 32 ? T : 32;

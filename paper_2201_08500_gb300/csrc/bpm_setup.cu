@@ -11,6 +11,7 @@
 #include <math.h>
 
 #include "bpm_internal.h"
+#include "bpm_norm.cuh"
 
 namespace bpm {
 
@@ -62,11 +63,6 @@ __device__ __forceinline__ float round_f32(double v) {
   const unsigned long long a = b & 0x7FFFFFFFFFFFFFFFull;
   const unsigned m = unsigned((a + 0x0FFFFFFFull + ((a >> 29) & 1)) >> 29) - (896u << 23);
   return __uint_as_float((a ? m : 0u) | (unsigned(b >> 32) & 0x80000000u));
-}
-__device__ __forceinline__ double widen_f64(float f) {
-  const unsigned b = __float_as_uint(f);
-  const unsigned long long a = ((unsigned long long)(b & 0x7FFFFFFFu) + (896ull << 23)) << 29;
-  return __longlong_as_double((long long)(a | ((unsigned long long)(b & 0x80000000u) << 32)));
 }
 // v as FP32 hi + lo, each rounded to nearest.
 __device__ __forceinline__ void split_f32(double v, float* hi, float* lo) {
