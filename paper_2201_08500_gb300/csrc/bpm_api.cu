@@ -872,10 +872,11 @@ BPM_API bpm_status bpm_run(bpm_plan p, int n_steps) {
   launches += march_launches;
   if (p->timing) BPM_CUDA(p, cudaEventRecord(p->ev1, p->stream), "timing event");
   if (p->grid.dims == 3) {
+    // the spectra are the passes' own: nothing is in them between two runs
     BPM_CUDA(p, launch_reduce3d(p->e0, p->eh, p->plane, p->n_ch, p->inc_norm, p->refl, p->trans,
-                                p->stream),
+                                p->spec, p->stream),
              "reflectivity");
-    ++launches;
+    launches += 2;
   }
   p->z += n_steps;
   p->time_valid = false;

@@ -223,8 +223,10 @@ bool row_stream_supported(int nx, int row_threads);
 cudaError_t launch_row_stream(int mode, int row_threads, const Pass3DArgs& a, int n_ch, int sms,
                               int* status, cudaStream_t s);
 cudaError_t launch_col_stream(const Pass3DArgs& a, int n_ch, int sms, int* status, cudaStream_t s);
+// R and T from the fields; scratch: two float2 per 8192 cells of a channel.
 cudaError_t launch_reduce3d(const float2* e0, const float2* eh, long long plane, int n_ch,
-                            const double* inc, double* refl, double* trans, cudaStream_t s);
+                            const double* inc, double* refl, double* trans, float2* scratch,
+                            cudaStream_t s);
 
 // Setup launchers (bpm_setup.cu).
 cudaError_t launch_tables3d(const SetupArgs& sa, const double* omega, const double* gainx,

@@ -12,10 +12,16 @@ __device__ __forceinline__ double widen_f64(float f) {
   const unsigned long long a = ((unsigned long long)(b & 0x7FFFFFFFu) + (896ull << 23)) << 29;
   return __longlong_as_double((long long)(a | ((unsigned long long)(b & 0x80000000u) << 32)));
 }
-// double(f) of any float.
+// double(f) of any float (a conversion for the rest, even one that no lane takes,
+// would hold the FP64 pipe all the same: sums over 128 planes of 512 x 512 513 -> 243 us).
 __device__ __forceinline__ double widen_any(float f) {
-  const unsigned e = __float_as_uint(f) & 0x7F800000u;
-  return e - 0x00800000u < 0x7F000000u ? widen_f64(f) : double(f);
+  const bool small = (__float_as_uint(f) & 0x7F800000u) == 0;  // zero or denormal
+  const float g = small ? f * 0x1p100f : f;
+  const unsigned b = __float_as_uint(g), m = b & 0x7FFFFFFFu;
+  unsigned long long a = ((unsigned long long)m + (small ? 796ull << 23 : 896ull << 23)) << 29;
+  if (m == 0) a = 0;
+  if (m >= 0x7F800000u) a |= 0x7FFull << 52;  // infinity, NaN
+  return __longlong_as_double((long long)(a | ((unsigned long long)(b & 0x80000000u) << 32)));
 }
 
 // s + |f|^2: two FP64 instructions (with conversions, a product and a separate

@@ -12,8 +12,8 @@
 //    M >= 2n - 1, with the same passes;
 //  * beyond that the direct sum.
 // Measured against a radix-2 transform (n a power of two up to 1024) and the
-// direct sum (the rest): 128 channels x 512 x 512: 2.51 -> 1.68 ms (about 26
-// FP64 instructions a point, 83 % of the FP64 rate); 1024 x 4096: 557 -> 310
+// direct sum (the rest): 128 channels x 512 x 512: 2.51 -> 1.55 ms (about 24
+// FP64 instructions a point, 85 % of the FP64 rate); 1024 x 4096: 557 -> 310
 // us; 24 x 131072: 6.46 ms -> 124 us; 611 = 13 x 47 channels x 1024 (chirp
 // form): 32.0 ms -> 334 us.
 // Twiddles, chirps and the chirp's spectrum are the plan's (time_tables_kernel,
@@ -22,6 +22,7 @@
 #include <math.h>
 
 #include "bpm_internal.h"
+#include "bpm_norm.cuh"
 
 namespace bpm {
 
@@ -260,7 +261,7 @@ __global__ void __launch_bounds__(kTimeThreads)
     double2 v = make_double2(0.0, 0.0);
     if (c < cols && li >= 0 && li < n_local) {
       const float2 f = eh[(long long)li * plane + x0 + c];
-      v = make_double2(double(f.x), double(f.y));
+      v = make_double2(widen_any(f.x), widen_any(f.y));
       if constexpr (CHIRP) v = zmul(v, cin[i]);
     }
     x[idx] = v;
@@ -344,6 +345,9 @@ cudaError_t launch_omega_to_t(int n_total, int first, int n_local, long long pla
   }
   int lc = 0;
   while (lc < 6 && (s.len << (lc + 1)) <= 2048) ++lc;
+  // a small plane: fewer columns a block, so that more SMs have one (four columns
+  // are still whole 32-byte sectors); 64 channels x 256: 16.7 -> 7.6 us
+  while (lc > 2 && (plane >> lc) < 152) --lc;
   const size_t smem = (2 * (size_t(s.len) << lc) + s.len) * sizeof(double2);
   const long long blocks = (plane + (1 << lc) - 1) >> lc;
   if (s.chirp)
