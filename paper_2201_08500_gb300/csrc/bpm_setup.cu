@@ -187,67 +187,84 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Power series of J0(w) and G1(w) = 2 J1(w)/w in terms of w^2 (A&S 9.1.10).
-// It ends where neither a term nor any later one (each at most half the one
-// before, once |z| <= k^2 / 2) can change a sum: after a few terms of the w of
-// thin slices, instead of a serial chain of 39 that took 80 us.
-__device__ void bessel_j0_g1(dc w2, dc* j0, dc* g1) {
+// Power series in w^2 of J0(w) (g1 = 0) or G1(w) = 2 J1(w)/w (g1 = 1) (A&S
+// 9.1.10).  It ends where neither a term nor any later one (each at most half the
+// one before, once |z| <= k^2 / 2) can change the sum: after a few terms of the w
+// of thin slices, instead of a serial chain of 39 that took 80 us.
+__device__ dc bessel_j0_g1(dc w2, int g1) {
   const dc z = dscale(w2, -0.25);
   const double az = fabs(z.re) + fabs(z.im);
-  dc t0 = dmk(1, 0), t1 = dmk(1, 0), s0 = dmk(1, 0), s1 = dmk(1, 0);
+  dc t = dmk(1, 0), s = dmk(1, 0);
   for (int k = 1; k < 40; ++k) {
-    t0 = ddiv_real(dmul(t0, z), double(k) * k);
-    t1 = ddiv_real(dmul(t1, z), double(k) * (k + 1));
-    s0 = dadd(s0, t0);
-    s1 = dadd(s1, t1);
-    const double tiny = (fabs(t0.re) + fabs(t0.im)) * 0x1p+54;
-    if (2.0 * az <= double(k) * k && tiny <= fabs(s0.re) && tiny <= fabs(s1.re) &&
-        (z.im == 0.0 || (tiny <= fabs(s0.im) && tiny <= fabs(s1.im))))
+    t = ddiv_real(dmul(t, z), double(k) * (k + g1));
+    s = dadd(s, t);
+    const double tiny = (fabs(t.re) + fabs(t.im)) * 0x1p+54;
+    if (2.0 * az <= double(k) * k && tiny <= fabs(s.re) && (z.im == 0.0 || tiny <= fabs(s.im)))
       break;
   }
-  *j0 = s0;
-  *g1 = s1;
+  return s;
 }
 
-// Coupling coefficients of Eq. fov10 for one channel: w^2 = (k dz / cos a)^2
-// chi_h chi_hbar, a = J0 e^{i phi} e^{w^2/8} (Zassenhaus), b+ = i G1 e^{i phi}
-// k dz chi_hbar / (2 cos a), b- likewise with chi_h; a split into hi + lo.
-__device__ ChannelCoef channel_coef(const SetupArgs& sa, double kdz, double cos_a) {
-  const dc chi0 = dmk(sa.chi0_re, sa.chi0_im);
-  const dc chih = dmk(sa.chih_re, sa.chih_im);
-  const dc chihb = dmk(sa.chihb_re, sa.chihb_im);
-  const double r = kdz / cos_a;
-  const dc w2 = dscale(dmul(chih, chihb), r * r);
-  const dc phase0 = dexp(dmul(dmk(0, 1), dscale(chi0, kdz / (2.0 * cos_a))));
-  dc j0, g1;
-  bessel_j0_g1(w2, &j0, &g1);
-  const dc zf = sa.zassenhaus ? dexp(dscale(w2, 0.125)) : dmk(1, 0);
-  const dc a = dmul(dmul(j0, phase0), zf);
-  const dc ig1p = dmul(dmk(0, 1), dmul(g1, phase0));
-  const dc bp = dmul(ig1p, dscale(chihb, kdz / (2.0 * cos_a)));
-  const dc bm = dmul(ig1p, dscale(chih, kdz / (2.0 * cos_a)));
-  ChannelCoef c;
-  c.a_hi = to_f2(a);
-  c.a_lo = make_float2(float(a.re - double(c.a_hi.x)), float(a.im - double(c.a_hi.y)));
-  c.bp = to_f2(bp);
-  c.bm = to_f2(bm);
-  return c;
+// The incident field needs nothing of the tables: its launch starts when all of
+// theirs run (programmatic dependent launch), and one block waits for them before
+// it ends, so that what follows the incident field follows both.
+__device__ __forceinline__ void after_tables() {
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void before_incident() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 constexpr int kTabThreads = 128;
 constexpr int kTabMaxCh = 8;  // channels per block of tables_kernel
 
-// Coupling coefficients of channel / set `i` (set fastest), fractions cfr of dz.
-__device__ void store_coef(const SetupArgs& sa, const double* omega, int i, int n_sets,
+// Coupling coefficients of Eq. fov10 for the 32 channels / sets from 32 `blk` on
+// (set fastest), fractions cfr of dz: w^2 = (k dz / cos a)^2 chi_h chi_hbar, a =
+// J0 e^{i phi} e^{w^2/8} (Zassenhaus), b+ = i G1 e^{i phi} k dz chi_hbar / (2 cos a),
+// b- likewise with chi_h; a split into hi + lo.  One lane an item, and a warp for
+// each of the four factors, chains of dependent FP64 instructions that took
+// 20 us one after the other, the whole kernel's time for a small plan.
+__device__ void store_coef(const SetupArgs& sa, const double* omega, int blk, int n_sets,
                            const double (&cfr)[2], ChannelCoef* coef, int* bad) {
-  const double k = omega[i / n_sets] / kC;
-  const double s_ratio = 0.5 * sa.h / k;
-  if (!(s_ratio < 1.0)) {
-    if (bad) atomicExch(bad, 1);
-    return;
+  __shared__ dc part[4][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = 32 * blk + lane;
+  double kdz = 0.0, cos_a = 1.0;
+  bool ok = i < sa.n_ch * n_sets;
+  if (ok) {
+    const double k = omega[i / n_sets] / kC;
+    const double s_ratio = 0.5 * sa.h / k;
+    ok = s_ratio < 1.0;
+    if (!ok && bad && w == 0) atomicExch(bad, 1);
+    cos_a = sqrt(1.0 - s_ratio * s_ratio);  // cos(alpha), Eq. fov3
+    kdz = k * sa.dz * cfr[i % n_sets];
   }
-  const double cos_a = sqrt(1.0 - s_ratio * s_ratio);  // cos(alpha), Eq. fov3
-  coef[i] = channel_coef(sa, k * sa.dz * cfr[i % n_sets], cos_a);
+  const dc chih = dmk(sa.chih_re, sa.chih_im), chihb = dmk(sa.chihb_re, sa.chihb_im);
+  if (ok) {
+    const double r = kdz / cos_a;
+    if (w == 2) {
+      const dc chi0 = dmk(sa.chi0_re, sa.chi0_im);
+      part[2][lane] = dexp(dmul(dmk(0, 1), dscale(chi0, kdz / (2.0 * cos_a))));
+    } else {
+      const dc w2 = dscale(dmul(chih, chihb), r * r);
+      part[w][lane] = w < 2            ? bessel_j0_g1(w2, w)
+                      : sa.zassenhaus ? dexp(dscale(w2, 0.125))
+                                      : dmk(1, 0);
+    }
+  }
+  __syncthreads();
+  if (!ok || w > 1) return;
+  const dc phase0 = part[2][lane];
+  if (w == 0) {
+    const dc a = dmul(dmul(part[0][lane], phase0), part[3][lane]);
+    const float2 hi = to_f2(a);
+    coef[i].a_hi = hi;
+    coef[i].a_lo = make_float2(float(a.re - double(hi.x)), float(a.im - double(hi.y)));
+  } else {
+    const dc ig1p = dmul(dmk(0, 1), dmul(part[1][lane], phase0));
+    const double half = kdz / (2.0 * cos_a);
+    coef[i].bp = to_f2(dmul(ig1p, dscale(chihb, half)));
+    coef[i].bm = to_f2(dmul(ig1p, dscale(chih, half)));
+  }
 }
 
 // Position of frequency bin f in the digit-reversed spectrum of n points: the
@@ -274,11 +291,11 @@ __device__ __forceinline__ int spectrum_position(int f, int n) {
 //  * a thread keeps its bin for up to kTabMaxCh channels: q and the gains'
 //    reciprocals are divided out once;
 //  * a grid of 128-bin blocks also spreads a single channel over many SMs, and
-//    the coefficients (a serial chain) run in blocks of their own in front, one
-//    thread per channel.
+//    the coefficients (serial chains) run in blocks of their own in front, a lane
+//    of four warps per channel.
 // 8192 bins x 512 channels: 1600 -> 771 us (about 100 FP64 instructions a pair
 // of entries); two sets of 4096 x 256: 660 -> 327 us; 48 plans of 512 x 1, one
-// after the other: 91 -> 20 us each.
+// after the other: 91 -> 11.6 us each (20 with the coefficients in one chain).
 __global__ void __launch_bounds__(kTabThreads)
     tables_kernel(SetupArgs sa, int coef_blocks, int cpb, const double* __restrict__ omega,
                   const double* __restrict__ gain, const int* __restrict__ rev, float4* tables,
@@ -286,14 +303,13 @@ __global__ void __launch_bounds__(kTabThreads)
   // fractions of dz of the propagations (tables) and couplings (coefficient
   // sets) of Eq. split-op: order 1: (1; 1); order 2: (1; 1/2); order 4:
   // (t, 1-2t; t/2, (1-t)/2) with t = 1/(2 - 2^(1/3))
+  before_incident();
   const double t4 = sa.split_order == 4 ? 1.0 / (2.0 - cbrt(2.0)) : 0.0;
   const int n_sets = sa.split_order == 4 ? 2 : 1;
   if (int(blockIdx.x) < coef_blocks) {
     const double cfr[2] = {sa.split_order == 4 ? 0.5 * t4 : (sa.split_order == 2 ? 0.5 : 1.0),
                            0.5 * (1.0 - t4)};
-    const int i = int(blockIdx.x) * 32 + threadIdx.x;
-    if (threadIdx.x < 32 && i < sa.n_ch * n_sets)
-      store_coef(sa, omega, i, n_sets, cfr, coef, bad);
+    store_coef(sa, omega, int(blockIdx.x), n_sets, cfr, coef, bad);
     return;
   }
   __shared__ double sk[kTabMaxCh];
@@ -343,10 +359,10 @@ __global__ void __launch_bounds__(kTabThreads)
     tables3d_kernel(SetupArgs sa, int coef_blocks, const double* __restrict__ omega,
                     const double* __restrict__ gainx, const int* __restrict__ revx, float4* anchor,
                     float* gcorr, ChannelCoef* coef) {
+  before_incident();
   if (int(blockIdx.x) < coef_blocks) {
     const double cfr[2] = {sa.coupling_frac, 0.0};
-    const int i = int(blockIdx.x) * 32 + threadIdx.x;
-    if (threadIdx.x < 32 && i < sa.n_ch) store_coef(sa, omega, i, 1, cfr, coef, nullptr);
+    store_coef(sa, omega, int(blockIdx.x), 1, cfr, coef, nullptr);
     return;
   }
   const int n = sa.nx, T = n / 16, chunks = n / kTabThreads;
@@ -392,12 +408,19 @@ __device__ __forceinline__ float narrow_f32(double v) {
 __device__ __forceinline__ dc denominator(const SetupArgs& sa) {
   return dmk(1.0, sa.zR != 0.0 ? sa.zx / sa.zR : 0.0);
 }
-// S times the square root of 1 / denominator (2D) or 1 / denominator (3D)
-__device__ __forceinline__ dc amplitude(const SetupArgs& sa, double2 w) {
+// Factors of all channels and cells: 1 / denominator, and its square root (2D) or
+// itself (3D), which S is multiplied by.  At the waist (denominator 1) they are
+// what the general formulas give, without their chains of divisions and roots.
+struct Beam {
+  dc inv_den, pref;
+};
+__device__ Beam beam_factors(const SetupArgs& sa) {
   const dc den = denominator(sa);
-  const dc pref = (sa.dims == 3) ? drecip(den) : drecip(dsqrt(den));
-  return dmul(dmk(w.x, w.y), pref);
+  if (den.im == 0.0) return Beam{dmk(1.0, -den.im), dmk(1.0, -den.im)};
+  const dc inv = drecip(den);
+  return Beam{inv, sa.dims == 3 ? inv : drecip(dsqrt(den))};
 }
+__device__ __forceinline__ dc amplitude(dc pref, double2 w) { return dmul(dmk(w.x, w.y), pref); }
 // g at the squared distance r2 from the beam's centre
 __device__ __forceinline__ dc gauss(const SetupArgs& sa, dc inv_den, double r2) {
   const double rr = r2 / (sa.w0 * sa.w0);
@@ -419,6 +442,7 @@ constexpr float kLogNormZero = -380.f;
 // Constants of a block's channels, one lane of the first warp each; below the
 // log|g| `least` no channel's value is above zero (-inf with a NaN amplitude).
 struct IncChannels {
+  Beam beam;
   dc sp[kIncMaxCh];
   double dq[kIncMaxCh];
   float bound[kIncMaxCh];
@@ -430,8 +454,10 @@ __device__ void load_channels(const SetupArgs& sa, const double* omega, const do
   if (c < nch) {
     const double k = omega[ch0 + c] / kC;
     s->dq[c] = k * sin(sa.theta_i) - 0.5 * sa.h;
-    s->sp[c] = amplitude(sa, weight[ch0 + c]);
+    const Beam beam = beam_factors(sa);
+    s->sp[c] = amplitude(beam.pref, weight[ch0 + c]);
     s->bound[c] = log_bound(s->sp[c]);
+    if (c == 0) s->beam = beam;
   }
   __syncthreads();
   if (c == 0) {
@@ -445,57 +471,53 @@ __device__ void load_channels(const SetupArgs& sa, const double* omega, const do
   __syncthreads();
 }
 
-// Sum over the block's 256 threads, in thread 0.
-__device__ double block_sum(double v, double* red) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+// The last of `blocks` blocks to leave their parts of the sum of |g|^2 adds the
+// `parts` parts, in an order that depends on their number alone, and writes every
+// channel's norm.
+__device__ void finish_norm(const SetupArgs& sa, const double2* weight, dc pref, int blocks,
+                            int parts, NormScratch* scratch, double* inc_norm) {
+  __shared__ int last;
+  __shared__ double total;
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = v;
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int w = 1; w < kIncThreads / 32; ++w) v += red[w];
-  return v;
-}
-
-// The last of `blocks` blocks to leave its part of the sum of |g|^2 adds the
-// parts in order and writes every channel's norm.
-__device__ void finish_norm(const SetupArgs& sa, const double2* weight, double part, int idx,
-                            int blocks, NormScratch* scratch, double* inc_norm, double* red) {
-  __shared__ bool last;
-  part = block_sum(part, red);
   if (threadIdx.x == 0) {
-    scratch->part[idx] = part;
     __threadfence();
     last = atomicAdd(&scratch->arrived, 1) == blocks - 1;
   }
   __syncthreads();
   if (!last) return;
   __threadfence();
-  double sum = 0.0;
-  for (int i = threadIdx.x; i < blocks; i += kIncThreads) sum += __ldcg(&scratch->part[i]);
-  sum = block_sum(sum, red);
-  if (threadIdx.x == 0) {
-    red[31] = sum;
-    scratch->arrived = 0;  // for the next pulse
+  if (threadIdx.x < 32) {
+    double sum = 0.0;
+    for (int i = threadIdx.x; i < parts; i += 32) sum += __ldcg(&scratch->part[i]);
+    for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+    if (threadIdx.x == 0) {
+      total = sum;
+      scratch->arrived = 0;  // for the next pulse
+    }
   }
   __syncthreads();
-  for (int c = threadIdx.x; c < sa.n_ch; c += kIncThreads) {
-    const dc sp = amplitude(sa, weight[c]);
-    inc_norm[c] = (sp.re * sp.re + sp.im * sp.im) * red[31];
+  for (int c = threadIdx.x; c < sa.n_ch; c += blockDim.x) {
+    const dc sp = amplitude(pref, weight[c]);
+    inc_norm[c] = (sp.re * sp.re + sp.im * sp.im) * total;
   }
 }
 
-// 2D: a block has 256 cells, one a thread, of up to kIncMaxCh channels.
-__global__ void __launch_bounds__(kIncThreads)
+// 2D: a block has THREADS cells, one a thread, of up to kIncMaxCh channels; the
+// norm's parts are of 32 cells.  A warp's FP64 instruction takes an SM 16 clocks, so
+// a small plan has blocks of 64: one channel of 512 points 21.4 -> 9.6 us (with
+// the beam's factors once a block, not once a thread), of which most is beside
+// the tables.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
     incident_kernel(SetupArgs sa, int cpb, const double* __restrict__ omega,
                     const double2* __restrict__ weight, float2* e0, float2* eh, double* inc_norm,
                     NormScratch* scratch) {
   __shared__ IncChannels sc;
-  __shared__ double red[32];
-  const int chunks = sa.nx / kIncThreads;
+  const int chunks = sa.nx / THREADS;
   const int ch0 = (int(blockIdx.x) / chunks) * cpb, nch = min(cpb, sa.n_ch - ch0);
-  const int chunk = int(blockIdx.x) % chunks, j = chunk * kIncThreads + threadIdx.x;
+  const int chunk = int(blockIdx.x) % chunks, j = chunk * THREADS + threadIdx.x;
   load_channels(sa, omega, weight, ch0, nch, &sc);
-  const dc inv_den = drecip(denominator(sa));
+  const dc inv_den = sc.beam.inv_den;
   const double x = double(j) * sa.dx, d = x - sa.x0, r2 = d * d;
   const float lg = log_gauss(sa, inv_den) * float(r2);
   dc g = dmk(0.0, 0.0);
@@ -511,8 +533,13 @@ __global__ void __launch_bounds__(kIncThreads)
     e0[size_t(ch0 + c) * sa.nx + j] = v;
     eh[size_t(ch0 + c) * sa.nx + j] = make_float2(0.f, 0.f);
   }
-  if (ch0 == 0)
-    finish_norm(sa, weight, g.re * g.re + g.im * g.im, chunk, chunks, scratch, inc_norm, red);
+  if (ch0 == 0) {
+    double part = g.re * g.re + g.im * g.im;
+    for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, off);
+    if (threadIdx.x % 32 == 0) scratch->part[j / 32] = part;
+    finish_norm(sa, weight, sc.beam.pref, chunks, sa.nx / 32, scratch, inc_norm);
+  }
+  after_tables();
 }
 
 // 3D: a block has a tile of kIncTile x kIncTile cells of up to kIncMaxCh
@@ -523,7 +550,7 @@ __global__ void __launch_bounds__(kIncThreads)
                       double* inc_norm, NormScratch* scratch) {
   __shared__ IncChannels sc;
   __shared__ dc ph[kIncMaxCh][kIncTile];
-  __shared__ double red[32];
+  __shared__ double red[kIncThreads / 32];
   const int tx = sa.nx / kIncTile, tiles = tx * (sa.ny / kIncTile);
   const int ch0 = (int(blockIdx.x) / tiles) * kIncMaxCh, nch = min(kIncMaxCh, sa.n_ch - ch0);
   const int tile = int(blockIdx.x) % tiles;
@@ -536,7 +563,7 @@ __global__ void __launch_bounds__(kIncThreads)
     ph[c][j] = dmk(co, s);
   }
   __syncthreads();
-  const dc inv_den = drecip(denominator(sa));
+  const dc inv_den = sc.beam.inv_den;
   const float lgs = log_gauss(sa, inv_den);
   const size_t plane = size_t(sa.nx) * sa.ny;
   // two neighbouring cells a thread: 32 threads a row of the tile
@@ -571,7 +598,17 @@ __global__ void __launch_bounds__(kIncThreads)
       *reinterpret_cast<float4*>(eh + at) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
-  if (ch0 == 0) finish_norm(sa, weight, acc, tile, tiles, scratch, inc_norm, red);
+  if (ch0 == 0) {
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < kIncThreads / 32; ++w) acc += red[w];
+      scratch->part[tile] = acc;
+    }
+    finish_norm(sa, weight, sc.beam.pref, tiles, tiles, scratch, inc_norm);
+  }
+  after_tables();
 }
 
 }  // namespace
@@ -614,20 +651,31 @@ cudaError_t launch_tables3d(const SetupArgs& sa, const double* omega, const doub
 cudaError_t launch_incident(const SetupArgs& sa, const double* omega, const double2* weight,
                             float2* e0, float2* eh, double* inc_norm, NormScratch* scratch,
                             cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.stream = s;
+  cudaLaunchAttribute at{};  // see after_tables
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
   if (sa.dims == 3) {
     const int tiles = (sa.nx / kIncTile) * (sa.ny / kIncTile);
     const int groups = (sa.n_ch + kIncMaxCh - 1) / kIncMaxCh;
-    incident3d_kernel<<<tiles * groups, kIncThreads, 0, s>>>(sa, omega, weight, e0, eh, inc_norm,
-                                                             scratch);
-    return cudaGetLastError();
+    cfg.gridDim = dim3(unsigned(tiles * groups));
+    cfg.blockDim = dim3(kIncThreads);
+    return cudaLaunchKernelEx(&cfg, incident3d_kernel, sa, omega, weight, e0, eh, inc_norm, scratch);
   }
-  // as in launch_tables: several channels a block once every SM has eight warps' work
-  const int chunks = sa.nx / kIncThreads;
+  // as in launch_tables: several channels a block once every SM has eight warps'
+  // work, and small blocks where that is not even so with one
+  int threads = kIncThreads;
+  auto blocks = [&](int cpb) { return sa.nx / threads * ((sa.n_ch + cpb - 1) / cpb); };
   int cpb = kIncMaxCh;
-  while (cpb > 1 && chunks * ((sa.n_ch + cpb - 1) / cpb) < 152 * 2) cpb /= 2;
-  incident_kernel<<<chunks * ((sa.n_ch + cpb - 1) / cpb), kIncThreads, 0, s>>>(
-      sa, cpb, omega, weight, e0, eh, inc_norm, scratch);
-  return cudaGetLastError();
+  while (cpb > 1 && blocks(cpb) < 152 * 2) cpb /= 2;
+  if (blocks(cpb) < 152 * 2) threads = 64;
+  cfg.gridDim = dim3(unsigned(blocks(cpb)));
+  cfg.blockDim = dim3(unsigned(threads));
+  return cudaLaunchKernelEx(&cfg, threads == 64 ? incident_kernel<64> : incident_kernel<kIncThreads>,
+                            sa, cpb, omega, weight, e0, eh, inc_norm, scratch);
 }
 
 }  // namespace bpm
