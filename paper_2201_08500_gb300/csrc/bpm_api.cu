@@ -250,8 +250,10 @@ struct bpm_plan_s {
   float2* twiddle_p = nullptr;   // 2D: the same in thread-ordered pairs
   int* rev = nullptr;
   double* gain = nullptr;
-  double* omega = nullptr;
+  // one copy each way: weights and then frequencies, R and then T
   double2* weight = nullptr;
+  double* omega = nullptr;
+  std::vector<double> pulse_host;  // the same, gathered for the copy
   double* inc_norm = nullptr;
   double* refl = nullptr;
   double* trans = nullptr;
@@ -318,8 +320,8 @@ cudaError_t dalloc(T** ptr, size_t count) {
 
 void free_plan_buffers(bpm_plan p) {
   void* ptrs[] = {p->cfield, p->e0,      p->eh,    p->tables, p->coef,     p->twiddle,
-                  p->rev,    p->gain,    p->omega, p->weight, p->inc_norm, p->refl,
-                  p->trans,  p->eh_time, p->dflag, p->u_tmp,  p->gcorr,    p->twy,
+                  p->rev,    p->gain,    p->weight, p->inc_norm, p->refl,
+                  p->eh_time, p->dflag,  p->u_tmp, p->gcorr,  p->twy,
                   p->qy,     p->spec,    p->twx3,  p->twiddle_t, p->twiddle_p, p->mask,
                   p->cspan,  p->time_tab, p->norm_scratch, p->ext};
   for (void* q : ptrs)
@@ -495,11 +497,11 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
   if (g.dims == 2) check(dalloc(&p->twiddle_p, 2 * size_t(g.nx)), "alloc paired twiddles");
   check(dalloc(&p->rev, size_t(g.nx)), "alloc spectrum order");
   check(dalloc(&p->gain, size_t(g.nx)), "alloc gain");
-  check(dalloc(&p->omega, size_t(n_channels)), "alloc omega");
-  check(dalloc(&p->weight, size_t(n_channels)), "alloc weights");
+  check(dalloc(&p->weight, size_t(n_channels) * 3 / 2 + 1), "alloc weights, omega");
+  p->omega = reinterpret_cast<double*>(p->weight + n_channels);
   check(dalloc(&p->inc_norm, size_t(n_channels)), "alloc norms");
-  check(dalloc(&p->refl, size_t(n_channels)), "alloc R");
-  check(dalloc(&p->trans, size_t(n_channels)), "alloc T");
+  check(dalloc(&p->refl, 2 * size_t(n_channels)), "alloc R, T");
+  p->trans = p->refl + n_channels;
   check(dalloc(&p->eh_time, nf), "alloc time response");
   check(dalloc(&p->time_tab, time_table_elems(n_channels)), "alloc time tables");
   const size_t n_flags = kHandoff + size_t(kSharesPerSm) * device_info().sm_count;
@@ -724,12 +726,25 @@ BPM_API bpm_status bpm_set_pulse(bpm_plan p, const double* omega, const double* 
   p->sa.zx = zx;
   p->sa.zR = zR;
   if (!p->sharded) p->domega = p->n_ch > 1 ? omega[1] - omega[0] : 1.0;
-  BPM_CUDA(p, cudaMemcpyAsync(p->omega, omega, sizeof(double) * p->n_ch, cudaMemcpyHostToDevice,
-                              p->stream),
-           "upload omega");
-  BPM_CUDA(p, cudaMemcpyAsync(p->weight, weight_re_im, sizeof(double2) * p->n_ch,
-                              cudaMemcpyHostToDevice, p->stream),
-           "upload weights");
+  const size_t n = size_t(p->n_ch);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  BPM_CUDA(p, cudaStreamIsCapturing(p->stream, &capture), "upload pulse");
+  if (capture == cudaStreamCaptureStatusNone) {
+    // one copy from pageable memory, which it has left when the call returns
+    p->pulse_host.resize(3 * n);
+    std::memcpy(p->pulse_host.data(), weight_re_im, 2 * n * sizeof(double));
+    std::memcpy(p->pulse_host.data() + 2 * n, omega, n * sizeof(double));
+    BPM_CUDA(p, cudaMemcpyAsync(p->weight, p->pulse_host.data(), 3 * n * sizeof(double),
+                                cudaMemcpyHostToDevice, p->stream),
+             "upload pulse");
+  } else {  // a replay copies what the caller's arrays then hold
+    BPM_CUDA(p, cudaMemcpyAsync(p->omega, omega, n * sizeof(double), cudaMemcpyHostToDevice,
+                                p->stream),
+             "upload omega");
+    BPM_CUDA(p, cudaMemcpyAsync(p->weight, weight_re_im, n * sizeof(double2),
+                                cudaMemcpyHostToDevice, p->stream),
+             "upload weights");
+  }
   BPM_CUDA(p, enqueue_pulse(p), "pulse setup kernels");
   p->have_pulse = true;
   return BPM_OK;
@@ -954,19 +969,17 @@ BPM_API bpm_status bpm_fetch_reflectivity(bpm_plan p, double* R, double* T, doub
   BPM_NVTX();
   if (!p) return fail(nullptr, BPM_ERR_INVALID_ARG, "null plan");
   if (!p->have_pulse) return fail(p, BPM_ERR_STATE, "no pulse set");
-  std::vector<double> r(p->n_ch), t(p->n_ch);
-  BPM_CUDA(p, cudaMemcpyAsync(r.data(), p->refl, sizeof(double) * p->n_ch, cudaMemcpyDeviceToHost,
+  const size_t n = size_t(p->n_ch);
+  std::vector<double> rt(2 * n);
+  BPM_CUDA(p, cudaMemcpyAsync(rt.data(), p->refl, 2 * n * sizeof(double), cudaMemcpyDeviceToHost,
                               p->stream),
-           "fetch R");
-  BPM_CUDA(p, cudaMemcpyAsync(t.data(), p->trans, sizeof(double) * p->n_ch,
-                              cudaMemcpyDeviceToHost, p->stream),
-           "fetch T");
+           "fetch R, T");
   BPM_CUDA(p, cudaStreamSynchronize(p->stream), "fetch reflectivity");
-  if (R) std::memcpy(R, r.data(), sizeof(double) * p->n_ch);
-  if (T) std::memcpy(T, t.data(), sizeof(double) * p->n_ch);
+  if (R) std::memcpy(R, rt.data(), n * sizeof(double));
+  if (T) std::memcpy(T, rt.data() + n, n * sizeof(double));
   if (R_int) {
     double s = 0.0;
-    for (double v : r) s += v;
+    for (size_t i = 0; i < n; ++i) s += rt[i];
     *R_int = p->domega * s;
   }
   return BPM_OK;
