@@ -8,14 +8,15 @@
 //  * n = 2^a 3^b 5^c 7^d (up to 4096): Stockham passes of radix 8, 4, 2, 3, 5
 //    and 7 through shared memory, about 3.3 FP64 instructions a point and
 //    octave (radix 2: 4, a direct sum: 4 n);
-//  * any other n up to 2048: Bluestein's chirp transform on the power of two
-//    M >= 2n - 1, with the same passes;
+//  * any other n up to 2048: Bluestein's chirp transform of the length M >= 2n - 1
+//    with the fewest operations, 2^a 3^b 5^c 7^d too, with the same passes (611
+//    channels: 1280, not 2048);
 //  * beyond that the direct sum.
 // Measured against a radix-2 transform (n a power of two up to 1024) and the
 // direct sum (the rest): 128 channels x 512 x 512: 2.51 -> 1.55 ms (about 24
 // FP64 instructions a point, 85 % of the FP64 rate); 1024 x 4096: 557 -> 310
 // us; 24 x 131072: 6.46 ms -> 124 us; 611 = 13 x 47 channels x 1024 (chirp
-// form): 32.0 ms -> 334 us.
+// form): 32.0 ms -> 236 us (334 at length 2048).
 // Twiddles, chirps and the chirp's spectrum are the plan's (time_tables_kernel,
 // written once for its n): made in each block they cost as much as a column.
 #include <cuda_runtime.h>
@@ -61,9 +62,27 @@ bool time_shape(int n, TimeShape* s) {
   if (n < 1) return false;
   s->n = s->len = n;
   if (n <= kTimeMaxLen && radices(n, s)) return true;
+  // the chirp form: of the odd parts, each with the power of two that it needs, the
+  // one with the fewest FP64 instructions
+  if (n > kTimeMaxLen / 2) return false;
   s->chirp = 1;
-  for (s->len = 1; s->len < 2 * n - 1 && s->len < kTimeMaxLen;) s->len *= 2;
-  return s->len >= 2 * n - 1 && radices(s->len, s);
+  double best = 0.0;
+  for (int odd : {1, 3, 5, 7, 9, 15, 21, 25, 27, 35, 45, 49}) {
+    TimeShape t = *s;
+    for (t.len = odd; t.len < 2 * n - 1;) t.len *= 2;
+    if (t.len > kTimeMaxLen || !radices(t.len, &t)) continue;
+    double cost = 0.0;
+    for (int p = 0; p < t.n_pass; ++p) {
+      const int r = t.radix[p];
+      cost += r == 8 ? 10.0 : r == 4 ? 7.0 : r == 2 ? 4.0 : r == 7 ? 12.9 : r == 5 ? 10.4 : 8.0;
+    }
+    cost *= t.len;
+    if (best == 0.0 || cost < best) {
+      best = cost;
+      *s = t;
+    }
+  }
+  return best > 0.0;
 }
 
 size_t time_table_elems(int n) {
@@ -233,7 +252,7 @@ __global__ void time_tables_kernel(TimeShape s, double2* tt) {
     if (i) x[s.len - i] = b;
   }
   const double2* f = time_passes(s, x, y, tw, 0);
-  const double inv = 1.0 / double(s.len);  // a power of two
+  const double inv = 1.0 / double(s.len);
   for (int i = threadIdx.x; i < s.len; i += blockDim.x)
     filt[i] = make_double2(f[i].x * inv, f[i].y * inv);
 }
@@ -344,7 +363,7 @@ cudaError_t launch_omega_to_t(int n_total, int first, int n_local, long long pla
     return cudaGetLastError();
   }
   int lc = 0;
-  while (lc < 6 && (s.len << (lc + 1)) <= 2048) ++lc;
+  while (lc < 6 && (s.len << (lc + 1)) <= 2560) ++lc;
   // a small plane: fewer columns a block, so that more SMs have one (four columns
   // are still whole 32-byte sectors); 64 channels x 256: 16.7 -> 7.6 us
   while (lc > 2 && (plane >> lc) < 152) --lc;
