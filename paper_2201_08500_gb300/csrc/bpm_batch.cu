@@ -192,12 +192,12 @@ __global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>
 // A resident item takes an SM for the time of a full one however few channels
 // it has (us a step, first order, Strang, fourth order: 256 points 2.9, 4.4,
 // 10.3; 512 points 4.7, 5.8, 15.6), a channel of the other form its share of
-// one (0.25, 0.275, 0.85; 0.65, 0.70, 2.29).  One kind for the whole round: the
+// one (0.25, 0.275, 0.85; 0.61, 0.66, 2.31).  One kind for the whole round: the
 // queues run one after the other.
 bool batch_singles(int n, int split_order, int channels, int items, int sms) {
   if (n > 512 || sms < 1) return false;
   const int i = n == 256 ? 0 : 1, o = split_order == 1 ? 0 : split_order == 2 ? 1 : 2;
-  static constexpr double each[2][3] = {{0.25, 0.275, 0.85}, {0.65, 0.70, 2.29}};
+  static constexpr double each[2][3] = {{0.25, 0.275, 0.85}, {0.61, 0.66, 2.31}};
   static constexpr double full[2][3] = {{2.9, 4.4, 10.3}, {4.7, 5.8, 15.6}};
   return each[i][o] * ((channels + sms - 1) / sms) < full[i][o] * ((items + sms - 1) / sms);
 }

@@ -42,19 +42,19 @@ int march_max_group(int n) {
 
 // Form and channels per block of a plan that names none, over 1 ... 2500
 // channels and 152 SMs (us a step, this form against the next best):
-//  * 256, 512 points: one channel a block while march_quad_use holds (1.45
-//    against 4.6 at 230 channels of 512), then at 256 sixteen (2.9 against 3.9
-//    at 2432);
-//  * 1024: one channel up to one an SM, fourth order and Strang up to two (1.8
-//    against 3.0 at 152 channels, 10.8 against 13.2 at 304); beyond, TMEM
-//    tables, two channels a block (3.0 against 3.6 at 230, 16.7 against 19.1 at
-//    2500), fourth order the parked form (18.7 against 23 at 611);
-//  * 2048: TMEM tables (4.06 against 4.41 at 152, 14.1 against 16.4 at 1024);
+//  * 256, 512 points: one channel a block while march_quad_use holds (3.1 against
+//    4.6 at 760 channels of 512), then at 256 sixteen (2.9 against 5.3 at 2000);
+//  * 1024: one channel a block up to 15/8 an SM, fourth order and Strang up to two
+//    (1.7 against 3.1 at 155 channels, 3.26 against 3.07 at 300; fourth order 10.5
+//    against 13.2 at 304); beyond, TMEM tables, two channels a block (3.1 against
+//    4.6 at 300, 16.7 against 19.1 at 2500), fourth order the parked form (18.7
+//    against 23 at 611);
+//  * 2048: TMEM tables (4.06 against 4.41 at 152, 13.2 against 16.4 at 1024);
 //    fourth order the parked form beyond two channels an SM (21.4 against 29.2
 //    at 456, but 16.4 against 16.1 at 304);
 //  * 4096: the resident form up to one channel an SM (5.1 against 5.4), then
-//    TMEM tables (8.8 against 9.8 at 230, 30.7 against 37.4 at 1024), fourth
-//    order parked (28.3 against 34.2 at 230);
+//    TMEM tables (7.9 against 9.8 at 230, 29.0 against 37.4 at 1024), fourth
+//    order parked (27.3 against 34.2 at 230);
 //  * 8192: TMEM tables (form 0 is the same kernel).
 void march_default_form(int n, int split_order, int n_ch, int sms, int* form, int* group) {
   *form = 0;
@@ -65,7 +65,7 @@ void march_default_form(int n, int split_order, int n_ch, int sms, int* form, in
       if (!march_quad_use(n, o, n_ch, sms)) *group = march_max_group(n);
       break;
     case 1024:
-      if (n_ch > (o == 1 ? sms : 2 * sms)) {
+      if (8 * n_ch > (o == 1 ? 15 : 16) * sms) {
         *form = o == 4 ? 2 : 3;
         *group = o == 4 ? 1 : 2;
       }
@@ -91,15 +91,15 @@ struct StepTimes {
   float t[8];
 };
 constexpr StepTimes kStepTimes[] = {
-    {256, 0, 1, {0.63f, 0.75f, 0.84f, 1.04f, 1.26f, 1.49f}},
-    {256, 0, 2, {0.92f, 1.02f, 1.10f, 1.26f, 1.46f, 1.64f}},
-    {256, 0, 4, {2.67f, 3.00f, 3.30f, 3.95f, 4.62f, 5.65f}},
-    {512, 0, 1, {1.05f, 1.44f, 1.95f}},
-    {512, 0, 2, {1.26f, 1.54f, 2.07f}},
-    {512, 0, 4, {3.77f, 5.12f, 7.32f}},
-    {1024, 0, 1, {1.79f}},
-    {1024, 0, 2, {1.97f}},
-    {1024, 0, 4, {5.40f}},
+    {256, 0, 1, {0.62f, 0.74f, 0.84f, 1.04f, 1.25f, 1.48f}},
+    {256, 0, 2, {0.92f, 1.01f, 1.11f, 1.25f, 1.43f, 1.64f}},
+    {256, 0, 4, {2.68f, 2.99f, 3.26f, 3.89f, 4.57f, 5.33f}},
+    {512, 0, 1, {0.98f, 1.35f, 1.83f}},
+    {512, 0, 2, {1.16f, 1.48f, 1.97f}},
+    {512, 0, 4, {3.73f, 5.29f, 6.94f}},
+    {1024, 0, 1, {1.64f}},
+    {1024, 0, 2, {1.84f}},
+    {1024, 0, 4, {5.24f}},
     {1024, 2, 1, {2.86f, 3.15f, 4.53f, 4.85f, 5.95f, 6.45f, 7.82f, 8.23f}},
     {1024, 2, 4, {9.46f, 12.1f, 14.8f, 15.7f, 18.9f, 20.2f, 24.2f, 25.4f}},
     {1024, 3, 1, {3.06f, 4.24f, 5.74f, 7.35f}},

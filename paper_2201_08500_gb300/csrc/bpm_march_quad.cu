@@ -32,13 +32,13 @@ cudaError_t launch_order(int blocks, const MarchArgs& a, cudaStream_t s) {
 
 // The step times of the forms for n_ch channels, in us (measured over 1 ... 2500
 // channels, 152 SMs).  Up to 3 (256, 512 points) or 1 (1024) channels an SM
-// this form ends in 0.7, 1.0 and 1.8 us; beyond, it takes its share of an SM's
+// this form ends in 0.6, 1.0 and 1.6 us; beyond, it takes its share of an SM's
 // time per channel, and the resident form a whole wave of 16, 8 or 4 channels
-// an SM whether full or not.  E.g. first order, 512 points: 201 channels 1.45
-// against 3.85, 760 3.7 against 4.05, 1024 4.5 against 4.2.
+// an SM whether full or not.  E.g. first order, 512 points: 201 channels 1.32
+// against 3.85, 760 3.1 against 4.05, 1024 4.1 against 4.2.
 bool march_quad_use(int n, int split_order, int n_ch, int sms) {
   const int o = split_order == 1 ? 0 : split_order == 2 ? 1 : 2;
-  static constexpr double each[3][3] = {{0.25, 0.275, 0.85}, {0.65, 0.70, 2.29}, {1.79, 1.97, 5.4}};
+  static constexpr double each[3][3] = {{0.25, 0.275, 0.85}, {0.61, 0.66, 2.31}, {1.64, 1.84, 5.24}};
   static constexpr double wave[3][3] = {{2.9, 4.35, 10.3}, {4.2, 5.2, 14.3}, {4.2, 5.2, 14.4}};
   if (n > 1024 || n_ch < 1 || sms < 1) return false;
   const int i = n == 256 ? 0 : n == 512 ? 1 : 2, per = n == 256 ? 16 : n == 512 ? 8 : 4;

@@ -15,10 +15,11 @@
 // bpm_resident.cuh, so the fields are bitwise the same, and so are the sums of
 // the reflectivity.
 //
-// A step of one channel, first order: 256 points 1.77 -> 0.69 us, 512 points
-// 3.1 ... 3.7 -> 1.04, 1024 points 3.2 ... 3.9 -> 1.77 (latency bound: six
-// barriers and the chains between them); 201 channels of 512 points 3.85 ->
-// 1.45; Strang 512 points 4.8 -> 1.26; fourth order 11.7 -> 3.76.
+// A step of one channel, first order: 256 points 1.77 -> 0.61 us, 512 points
+// 3.1 ... 3.7 -> 0.97, 1024 points 3.2 ... 3.9 -> 1.62 (latency bound: six
+// barriers and the chains between them; an SM issues in 22 to 38 % of its
+// cycles); 201 channels of 512 points 3.85 -> 1.32; Strang 512 points 4.8 -> 1.15;
+// fourth order 11.7 -> 3.7.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -107,9 +108,11 @@ struct Quad {
     return make_float2(__shfl_xor_sync(0xFFFFFFFFu, v.x, mask),
                        __shfl_xor_sync(0xFFFFFFFFu, v.y, mask));
   }
-  // own + other, or other - own in the upper lane of a pair
-  static BPM_DEV float2 sumdiff(float2 own, float2 other, bool upper) {
-    return upper ? c_sub(other, own) : c_add(own, other);
+  // own + other, or (sign -1: the upper lane of a pair) other - own: one rounding
+  // either way, and one instruction instead of two and a selection (512 points 1.05
+  // -> 0.97 us a step, 1024 points 1.79 -> 1.68).
+  static BPM_DEV float2 sumdiff(float2 own, float2 other, float sign) {
+    return c_fmas(own, sign, other);
   }
 
   // Last stage over the RL lanes that share a block of positions (t % RL).
@@ -119,7 +122,7 @@ struct Quad {
   static BPM_DEV void last(float2 (&v)[4], int t) {
     if constexpr (RL == 2) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = sumdiff(v[i], shfl(v[i], 1), t & 1);
+      for (int i = 0; i < 4; ++i) v[i] = sumdiff(v[i], shfl(v[i], 1), t & 1 ? -1.f : 1.f);
     } else if constexpr (RL == 4) {
       // forward: sums and differences of lanes 2 apart, then of neighbours;
       // inverse: the other way round.  The pair of differences combines with
@@ -129,10 +132,10 @@ struct Quad {
       const float sg = (upper != INV) ? -1.f : 1.f;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float2 a = sumdiff(v[i], shfl(v[i], m0), t & m0);
+        const float2 a = sumdiff(v[i], shfl(v[i], m0), turned ? -1.f : 1.f);
         const float2 o = shfl(a, m1);
         const float2 d0 = upper ? o : a, d1 = upper ? a : o;
-        const float2 plain = sumdiff(a, o, upper);
+        const float2 plain = sumdiff(a, o, upper ? -1.f : 1.f);
         const float2 quarter = make_float2(fmaf(d1.y, sg, d0.x), fmaf(-d1.x, sg, d0.y));
         v[i] = turned ? quarter : plain;
       }
@@ -142,18 +145,22 @@ struct Quad {
     return RL == 4 ? (t & ~3) | ((t & 1) << 1) | ((t >> 1) & 1) : t;
   }
 
+  // The product by the twiddle of k = 0, which is one, too: at 1024 points cheaper than
+  // the branch around it (1.68 -> 1.62 us a step; 512 points 0.97 -> 1.00).
+  static constexpr bool kMulAll = N == 1024;
+
   // Forward FFT, propagator (table set s), inverse FFT of the thread's envelope.
   static BPM_DEV void propagate(float2 (&v)[4], const Ctx& c, int s) {
     dft16<false>(v, c.x0, c.t, c.q);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      if (i > 0 || c.q > 0) v[i] = c_mul(v[i], c.tw0[i]);
+      if (kMulAll || i > 0 || c.q > 0) v[i] = c_mul(v[i], c.tw0[i]);
     xchg16<false>(v, c.x1, c.t, c.q);
     dft16<false>(v, c.x0, c.t, c.q);
     if constexpr (RL > 1) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        if (i > 0 || c.q > 0) v[i] = c_mul(v[i], c.tw1[i]);
+        if (kMulAll || i > 0 || c.q > 0) v[i] = c_mul(v[i], c.tw1[i]);
     }
     last<false>(v, c.t);
 #pragma unroll
@@ -162,13 +169,13 @@ struct Quad {
     if constexpr (RL > 1) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        if (i > 0 || c.q > 0) v[i] = c_mulc(v[i], c.tw1[i]);
+        if (kMulAll || i > 0 || c.q > 0) v[i] = c_mulc(v[i], c.tw1[i]);
     }
     dft16<true>(v, c.x1, c.t, c.q);
     xchg16<true>(v, c.x0, c.t, c.q);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      if (i > 0 || c.q > 0) v[i] = c_mulc(v[i], c.tw0[i]);
+      if (kMulAll || i > 0 || c.q > 0) v[i] = c_mulc(v[i], c.tw0[i]);
     dft16<true>(v, c.x1, c.t, c.q);
   }
 
