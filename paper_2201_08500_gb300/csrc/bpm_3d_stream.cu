@@ -170,6 +170,34 @@ struct FftL {
   }
 };
 
+// Passes of a run after the first are programmatic dependents of the pass before:
+// their blocks start in its empty end, set themselves up and wait here for it to
+// complete (and with it, in turn, every earlier one).  That hides a launch's 2 us
+// where the passes are short: us a step 256 x 256 x 1 channel 10.3 -> 8.4, 256 x 512
+// x 8 24.7 -> 20.2, 256 x 256 x 64 57.7 -> 53.6, 1024 x 512 x 16 152.3 -> 149.5, 512 x
+// 512 x 64 227.0 -> 225.4 (256 x 512 x 24 47.6 -> 48.1: its grids leave no room to start
+// in).
+BPM_DEV void pass_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... Params, typename... Args>
+cudaError_t launch_pass(void (*kernel)(Params...), int blocks, int threads, size_t smem, bool follow,
+                        cudaStream_t s, const Args&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(blocks));
+  cfg.blockDim = dim3(unsigned(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = follow ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Column pass: each group of 2 TH lanes walks its share of the n_ch nx columns
 // (both envelopes of one, 16 NY contiguous bytes): forward y, propagator,
 // inverse y, in place.  A bulk copy brings the next column into the group's
@@ -210,8 +238,9 @@ __global__ void __launch_bounds__(ColStream<NY>::kBlock, ColStream<NY>::kBlocksP
   if (l == 0) {
     mbar_init(bar, 1);
     mbar_init_fence();
-    if (col < n_cols) issue(col);
   }
+  pass_begin();
+  if (l == 0 && col < n_cols) issue(col);
   F::sync(g);
   uint32_t phase = 0;
   for (; col < n_cols; col += stride) {
@@ -354,8 +383,9 @@ __global__ void __launch_bounds__(RowStream<NX, R>::kBlock, RowStream<NX, R>::kB
   if (MODE != 0 && threadIdx.x == 0) {
     mbar_init(bar, 1);
     mbar_init_fence();
-    if (tile < n_tiles) issue(tile);
   }
+  pass_begin();
+  if (MODE != 0 && threadIdx.x == 0 && tile < n_tiles) issue(tile);
   __syncthreads();
   uint32_t phase = 0;
   for (; tile < n_tiles; tile += gridDim.x) {
@@ -495,13 +525,10 @@ cudaError_t row_launch(int mode, const Pass3DArgs& a, int n_ch, int sms, int* st
   const long long tiles = (long long)n_ch * (a.ny / R), cap = (long long)sms * L::kBlocksPerSm;
   const int blocks = int(tiles < cap ? tiles : cap);
   if (blocks == 0) return cudaSuccess;
-  if (mode == 0)
-    row_stream_kernel<NX, R, 0><<<blocks, L::kBlock, L::kSmem, s>>>(m, a, n_ch, status);
-  else if (mode == 1)
-    row_stream_kernel<NX, R, 1><<<blocks, L::kBlock, L::kSmem, s>>>(m, a, n_ch, status);
-  else
-    row_stream_kernel<NX, R, 2><<<blocks, L::kBlock, L::kSmem, s>>>(m, a, n_ch, status);
-  return cudaGetLastError();
+  auto* kernel = mode == 0   ? row_stream_kernel<NX, R, 0>
+                 : mode == 1 ? row_stream_kernel<NX, R, 1>
+                             : row_stream_kernel<NX, R, 2>;
+  return launch_pass(kernel, blocks, L::kBlock, L::kSmem, mode != 0, s, m, a, n_ch, status);
 }
 
 template <int NY>
@@ -509,8 +536,8 @@ cudaError_t col_launch(const Pass3DArgs& a, int n_ch, int sms, int* status, cuda
   using C = ColStream<NY>;
   const long long need = ((long long)n_ch * a.nx + C::G - 1) / C::G;
   const long long cap = (long long)sms * C::kBlocksPerSm;
-  col_stream_kernel<NY><<<int(need < cap ? need : cap), C::kBlock, C::kSmem, s>>>(a, n_ch, status);
-  return cudaGetLastError();
+  return launch_pass(col_stream_kernel<NY>, int(need < cap ? need : cap), C::kBlock, C::kSmem, true, s,
+                     a, n_ch, status);
 }
 
 template <int NX, int R>
