@@ -500,7 +500,7 @@ def run_3d(args, world, rank, local, jobs=None):
                      "algorithmic_bytes": 64 * w.n_ch * w.plane,
                      "kernel": {0: "row_pass_kernel + col_pass_kernel",
                                 1: "row_pass_kernel + col_pass_tma_kernel",
-                                2: "row_pass_tma_kernel + col_pass_tma_kernel"}[launch["form"]]
+                                2: "row_stream_kernel + col_stream_kernel"}[launch["form"]]
                                + " (2 passes per z step)",
                      "bytes_per_cell_update": 64, "march_ms": march_ms,
                      "passes": st["march_launches"]},
