@@ -242,12 +242,12 @@ cudaError_t launch_deformation(const SetupArgs& sa, const double* u_dev, float2*
 cudaError_t launch_tables(const SetupArgs& sa, const double* omega, const double* gain,
                           const int* rev, float4* tables, ChannelCoef* coef, int* bad,
                           cudaStream_t s);
-// Parts of the incident field's norm (one per 32 cells in 2D, per 64 x 64 in
+// Parts of the incident field's norm (one per 32 cells in 2D, per 64 x 16 in
 // 3D) and the count of blocks that have written theirs: zero before the first
 // launch, and again after each.
 struct NormScratch {
   int arrived;
-  double part[256];
+  double part[1024];
 };
 // Follows launch_tables or launch_tables3d on the stream, and may start before
 // they end (they share nothing); done when both are.

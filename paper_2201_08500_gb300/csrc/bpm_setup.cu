@@ -398,7 +398,8 @@ __global__ void __launch_bounds__(kTabThreads)
 // 256 x 512 x 24: 3.71 ms -> 165 us.
 constexpr int kIncThreads = 256;
 constexpr int kIncMaxCh = 8;
-constexpr int kIncTile = 64;   // 3D: cells of a block in x and in y
+constexpr int kIncTile = 64;   // 3D: cells of a block in x
+constexpr int kIncRows = 16;   // and in y
 
 __device__ __forceinline__ float narrow_f32(double v) {
   const unsigned e = (unsigned(__double_as_longlong(v) >> 52)) & 0x7FFu;
@@ -542,8 +543,12 @@ __global__ void __launch_bounds__(THREADS)
   after_tables();
 }
 
-// 3D: a block has a tile of kIncTile x kIncTile cells of up to kIncMaxCh
-// channels, the phases of its columns in shared memory.
+// 3D: a block has a tile of kIncTile x kIncRows cells of up to kIncMaxCh channels,
+// the phases of its columns in shared memory.  The beam fills a few tiles and the
+// rest is written as zeros, without phases; the low tiles spread the beam's FP64
+// work over the SMs (64 rows: the few blocks with the beam took 150 us each, two or
+// three of them on an SM).  512 x 512 x 128 channels 490 -> 293 us, 256 x 512 x 24
+// 165 -> 106.
 __global__ void __launch_bounds__(kIncThreads)
     incident3d_kernel(SetupArgs sa, const double* __restrict__ omega,
                       const double2* __restrict__ weight, float2* e0, float2* eh,
@@ -551,11 +556,38 @@ __global__ void __launch_bounds__(kIncThreads)
   __shared__ IncChannels sc;
   __shared__ dc ph[kIncMaxCh][kIncTile];
   __shared__ double red[kIncThreads / 32];
-  const int tx = sa.nx / kIncTile, tiles = tx * (sa.ny / kIncTile);
+  const int tx = sa.nx / kIncTile, tiles = tx * (sa.ny / kIncRows);
   const int ch0 = (int(blockIdx.x) / tiles) * kIncMaxCh, nch = min(kIncMaxCh, sa.n_ch - ch0);
   const int tile = int(blockIdx.x) % tiles;
-  const int jt = (tile % tx) * kIncTile, rt = (tile / tx) * kIncTile;
+  const int jt = (tile % tx) * kIncTile, rt = (tile / tx) * kIncRows;
   load_channels(sa, omega, weight, ch0, nch, &sc);
+  const size_t plane = size_t(sa.nx) * sa.ny;
+  // two neighbouring cells a thread: 32 threads a row of the tile
+  const int jj = 2 * (threadIdx.x % (kIncTile / 2));
+  const float lgs = log_gauss(sa, sc.beam.inv_den);
+  const float least = ch0 == 0 ? fminf(sc.least, kLogNormZero) : sc.least;
+  // no cell of the tile is nearer to the beam's centre than this, and rounding
+  // keeps the order
+  auto nearest = [](double lo, double hi, double at) {
+    return at < lo ? lo - at : at > hi ? hi - at : 0.0;
+  };
+  const double dx0 = nearest(double(jt) * sa.dx, double(jt + kIncTile - 1) * sa.dx, sa.x0);
+  const double dy0 = nearest((double(rt) - double(sa.ny / 2)) * sa.dy,
+                             (double(rt + kIncRows - 1) - double(sa.ny / 2)) * sa.dy, 0.0);
+  if (lgs <= 0.f && lgs * float(dx0 * dx0 + dy0 * dy0) < least) {
+    for (int r = threadIdx.x / (kIncTile / 2); r < kIncRows; r += kIncThreads / (kIncTile / 2))
+      for (int c = 0; c < nch; ++c) {
+        const size_t at = size_t(ch0 + c) * plane + size_t(rt + r) * sa.nx + jt + jj;
+        *reinterpret_cast<float4*>(e0 + at) = make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(eh + at) = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    if (ch0 == 0) {
+      if (threadIdx.x == 0) scratch->part[tile] = 0.0;
+      finish_norm(sa, weight, sc.beam.pref, tiles, tiles, scratch, inc_norm);
+    }
+    after_tables();
+    return;
+  }
   for (int i = threadIdx.x; i < nch * kIncTile; i += kIncThreads) {
     const int c = i / kIncTile, j = i % kIncTile;
     double s, co;
@@ -564,12 +596,8 @@ __global__ void __launch_bounds__(kIncThreads)
   }
   __syncthreads();
   const dc inv_den = sc.beam.inv_den;
-  const float lgs = log_gauss(sa, inv_den);
-  const size_t plane = size_t(sa.nx) * sa.ny;
-  // two neighbouring cells a thread: 32 threads a row of the tile
-  const int jj = 2 * (threadIdx.x % (kIncTile / 2));
   double acc = 0.0;
-  for (int r = threadIdx.x / (kIncTile / 2); r < kIncTile; r += kIncThreads / (kIncTile / 2)) {
+  for (int r = threadIdx.x / (kIncTile / 2); r < kIncRows; r += kIncThreads / (kIncTile / 2)) {
     const double y = (double(rt + r) - double(sa.ny / 2)) * sa.dy;
     dc g[2];
     float lg[2];
@@ -579,8 +607,7 @@ __global__ void __launch_bounds__(kIncThreads)
       const double r2 = (x - sa.x0) * (x - sa.x0) + y * y;
       lg[h] = lgs * float(r2);
       g[h] = dmk(0.0, 0.0);
-      if (!(lg[h] < (ch0 == 0 ? fminf(sc.least, kLogNormZero) : sc.least)))
-        g[h] = gauss(sa, inv_den, r2);
+      if (!(lg[h] < least)) g[h] = gauss(sa, inv_den, r2);
       acc += g[h].re * g[h].re + g[h].im * g[h].im;
     }
     for (int c = 0; c < nch; ++c) {
@@ -659,7 +686,7 @@ cudaError_t launch_incident(const SetupArgs& sa, const double* omega, const doub
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   if (sa.dims == 3) {
-    const int tiles = (sa.nx / kIncTile) * (sa.ny / kIncTile);
+    const int tiles = (sa.nx / kIncTile) * (sa.ny / kIncRows);
     const int groups = (sa.n_ch + kIncMaxCh - 1) / kIncMaxCh;
     cfg.gridDim = dim3(unsigned(tiles * groups));
     cfg.blockDim = dim3(kIncThreads);
