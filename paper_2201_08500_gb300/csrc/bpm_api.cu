@@ -837,7 +837,10 @@ BPM_API bpm_status bpm_run(bpm_plan p, int n_steps) {
     const int sms = device_info().sm_count;
     a.per_sm = march_shares(p->grid.nx, a.split_order, form, group, p->n_ch, n_steps, sms);
     a.handoff = p->dflag + kHandoff;
-    if (a.per_sm) p->stats.blocks = p->blocks = a.per_sm * sms;
+    if (a.per_sm) {
+      p->stats.blocks = p->blocks = a.per_sm * sms;
+      p->stats.smem_bytes = int(share_smem(size_t(p->stats.smem_bytes), a.per_sm));
+    }
     if (form == 1 && a.split_order == 1)
       BPM_CUDA(p, launch_march_l2(p->grid.nx, group, p->blocks, a, p->stream), "march kernel");
     else if ((form == 2 && a.split_order != 2) || (form == 3 && a.split_order <= 2))

@@ -179,6 +179,13 @@ cudaError_t march_set_attributes_quad();
 int march_shares(int n, int split_order, int form, int group, int n_ch, int n_steps, int sms);
 // Marks a plan keeps for it: one a slot.
 constexpr int kSharesPerSm = 8;
+// Dynamic shared memory that leaves room for `per_sm` blocks on an SM and not
+// one more (228 KB an SM, 1 KB of it a block's own): the grid of a shared march
+// is per_sm blocks an SM, and the hardware fills an SM before it takes the next.
+constexpr size_t share_smem(size_t need, int per_sm) {
+  const size_t least = per_sm > 0 ? (size_t(228) << 10) / size_t(per_sm + 1) - 512 : 0;
+  return need > least ? need : least;
+}
 // Second form of the first-order march: propagator tables and stage twiddles
 // read from L2 instead of shared memory / registers, at most 128 registers, so
 // that two blocks (two channel groups at independent FFT phases) share an SM.

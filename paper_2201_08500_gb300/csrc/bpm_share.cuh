@@ -83,12 +83,4 @@ __device__ __forceinline__ void share_next(const MarchArgs& A, int slot, int slo
   share_next(s, slot, slots, A.n_ch, A.z0, A.n_steps, A.per_sm, A.handoff);
 }
 
-// Dynamic shared memory that leaves room for `per_sm` blocks on an SM and not
-// one more (228 KB an SM, 1 KB of it a block's own): the grid of a shared march
-// is per_sm blocks an SM, and the hardware fills an SM before it takes the next.
-constexpr size_t share_smem(size_t need, int per_sm) {
-  const size_t least = per_sm > 0 ? (size_t(228) << 10) / size_t(per_sm + 1) - 512 : 0;
-  return need > least ? need : least;
-}
-
 }  // namespace bpm
