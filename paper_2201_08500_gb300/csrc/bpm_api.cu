@@ -379,9 +379,12 @@ void apply_launch(bpm_plan p, int form, int group) {
   const int nx = p->grid.nx;
   const bool quad = form == 0 && group == 1 &&
                     march_quad_use(nx, p->grid.split_order, p->n_ch, device_info().sm_count);
-  p->stats.threads_per_channel = quad ? 8 * (nx / 16) : march_threads_per_channel(nx);
+  const bool dual = form == 0 && group == 1 &&
+                    march_dual_use(nx, p->grid.split_order, p->n_ch, device_info().sm_count);
+  p->stats.threads_per_channel = (quad ? 8 : dual ? 2 : 1) * march_threads_per_channel(nx);
   p->stats.blocks = p->blocks;
   p->stats.smem_bytes = int(quad        ? march_quad_smem_bytes(nx)
+                            : dual      ? march_dual_smem_bytes(nx)
                             : form == 1 ? march_l2_smem_bytes(nx, group)
                             : form >= 2 ? march_parked_smem_bytes(nx, form)
                                         : march_smem_bytes(nx, group));

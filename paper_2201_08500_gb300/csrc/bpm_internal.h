@@ -174,6 +174,11 @@ bool march_quad_use(int n, int split_order, int n_ch, int sms);
 size_t march_quad_smem_bytes(int n);
 cudaError_t launch_march_quad(int n, int blocks, const MarchArgs& a, cudaStream_t s);
 cudaError_t march_set_attributes_quad();
+// The march with 2 n/16 threads a channel (bpm_march_dual.cu), n = 2048, likewise.
+bool march_dual_use(int n, int split_order, int n_ch, int sms);
+size_t march_dual_smem_bytes(int n);
+cudaError_t launch_march_dual(int n, int blocks, const MarchArgs& a, cudaStream_t s);
+cudaError_t march_set_attributes_dual();
 // Blocks an SM of a march in equal shares (bpm_share.cuh), 0 for one channel a
 // group in turn.
 int march_shares(int n, int split_order, int form, int group, int n_ch, int n_steps, int sms);

@@ -49,7 +49,8 @@ int march_max_group(int n) {
 //    against 13.2 at 304); beyond, TMEM tables, two channels a block (3.1 against
 //    4.6 at 300, 16.7 against 19.1 at 2500), fourth order the parked form (18.7
 //    against 23 at 611);
-//  * 2048: TMEM tables (4.06 against 4.41 at 152, 13.2 against 16.4 at 1024);
+//  * 2048: one channel a block while march_dual_use holds (2.6 against 4.1 at 152),
+//    then TMEM tables (13.2 against 16.4 at 1024);
 //    fourth order the parked form beyond two channels an SM (21.4 against 29.2
 //    at 456, but 16.4 against 16.1 at 304);
 //  * 4096: the resident form up to one channel an SM (5.1 against 5.4), then
@@ -71,6 +72,7 @@ void march_default_form(int n, int split_order, int n_ch, int sms, int* form, in
       }
       break;
     case 2048:
+      if (march_dual_use(n, o, n_ch, sms)) break;
       if (o != 4)
         *form = 3;
       else if (n_ch > 2 * sms)
@@ -87,7 +89,7 @@ namespace {
 
 // us a step with k = 1, 2, ... blocks on every SM (as many as fit), 152 SMs.
 struct StepTimes {
-  int n, form, order;  // form 0: bpm_quad.cuh
+  int n, form, order;  // form 0: bpm_quad.cuh, bpm_dual.cuh
   float t[8];
 };
 constexpr StepTimes kStepTimes[] = {
@@ -104,6 +106,9 @@ constexpr StepTimes kStepTimes[] = {
     {1024, 2, 4, {9.46f, 12.1f, 14.8f, 15.7f, 18.9f, 20.2f, 24.2f, 25.4f}},
     {1024, 3, 1, {3.06f, 4.24f, 5.74f, 7.35f}},
     {1024, 3, 2, {3.92f, 4.83f, 6.40f, 8.29f}},
+    {2048, 0, 1, {2.64f}},
+    {2048, 0, 2, {3.28f}},
+    {2048, 0, 4, {8.40f}},
     {2048, 2, 1, {4.12f, 5.30f, 6.85f, 8.71f}},
     {2048, 2, 4, {13.8f, 16.0f, 21.7f, 27.4f}},
     {2048, 3, 1, {4.11f, 4.46f, 6.18f, 7.97f}},
@@ -132,7 +137,10 @@ constexpr StepTimes kStepTimes[] = {
 int march_shares(int n, int split_order, int form, int group, int n_ch, int n_steps, int sms) {
   if (n == 8192) form = 0;
   if (n_steps < 16 || sms < 1 || form == 1) return 0;
-  if (form == 0 && n != 8192 && (group != 1 || !march_quad_use(n, split_order, n_ch, sms))) return 0;
+  if (form == 0 && n != 8192 &&
+      (group != 1 || !(march_quad_use(n, split_order, n_ch, sms) ||
+                       march_dual_use(n, split_order, n_ch, sms))))
+    return 0;
   const StepTimes* s = nullptr;
   for (const StepTimes& row : kStepTimes)
     if (row.n == n && row.form == form && row.order == split_order) s = &row;
@@ -163,6 +171,7 @@ cudaError_t march_set_attributes() {
   cudaError_t e = march_set_attributes_strang();
   if (cudaError_t e4 = march_set_attributes_split4(); e4 != cudaSuccess) e = e4;
   if (cudaError_t eq = march_set_attributes_quad(); eq != cudaSuccess) e = eq;
+  if (cudaError_t ed = march_set_attributes_dual(); ed != cudaSuccess) e = ed;
   cudaError_t r[] = {attr_one<256, 1, 1>(),  attr_one<256, 16, 1>(),
                      attr_one<512, 1, 1>(),  attr_one<512, 8, 1>(),
                      attr_one<1024, 1, 1>(), attr_one<1024, 4, 1>(),
@@ -177,6 +186,9 @@ cudaError_t launch_march(int n, int group, int blocks, const MarchArgs& a, cudaS
   int sms = 0;
   if (group == 1 && device_ready(&sms) && march_quad_use(n, a.split_order, a.n_ch, sms))
     return launch_march_quad(n, blocks, a, s);
+  if (group == 1 && sms > 0 && a.ext && a.twiddle_p &&  // (not the allocation-free entry)
+      march_dual_use(n, a.split_order, a.n_ch, sms))
+    return launch_march_dual(n, blocks, a, s);
   if (a.split_order == 2) return launch_march_strang(n, group, blocks, a, s);
   if (a.split_order == 4) return launch_march_split4(n, group, blocks, a, s);
 #define BPM_LAUNCH_CASE(NN, GG) \

@@ -24,6 +24,7 @@
 
 #include <cuda_runtime.h>
 
+#include "bpm_half.cuh"
 #include "bpm_norm.cuh"
 #include "bpm_resident.cuh"
 #include "bpm_share.cuh"
@@ -179,24 +180,7 @@ struct Quad {
     dft16<true>(v, c.x1, c.t, c.q);
   }
 
-  // Coefficients of one envelope's half of the coupling: own <- a own + b c' other,
-  // c' = c for E0 and conj(c) for Eh (couple_cell's operations).
-  struct Half {
-    float2 ah, al;
-    float bx, r1, py, r2;
-  };
-  static BPM_DEV Half half(const ChannelCoef& cf, int env) {
-    const float2 b = env ? cf.bm : cf.bp;
-    Half h;
-    h.ah = cf.a_hi;
-    h.al = cf.a_lo;
-    h.bx = b.x;
-    h.r1 = env ? b.y : -b.y;
-    h.py = env ? b.y : b.x;
-    h.r2 = env ? -b.x : b.y;
-    return h;
-  }
-  static BPM_DEV void couple(float2 (&v)[4], const float2 (&cc)[4], const Half& h, int env) {
+  static BPM_DEV void couple(float2 (&v)[4], const float2 (&cc)[4], const HalfCoef& h, int env) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       // both halves of the warp hold the same cells: the vote keeps the shuffles whole
@@ -204,14 +188,7 @@ struct Quad {
       if (!__any_sync(0xFFFFFFFFu, in)) continue;
       const float2 o = shfl(v[i], 16);
       if (!in) continue;
-      const float2 c = cc[i], p = v[i];
-      const float2 bc = make_float2(fmaf(h.bx, c.x, h.r1 * c.y),
-                                    fmaf(h.py, env ? c.x : c.y, h.r2 * (env ? c.y : c.x)));
-      v[i] = make_float2(
-          fmaf(h.ah.x, p.x, fmaf(-h.ah.y, p.y, fmaf(bc.x, o.x, fmaf(-bc.y, o.y,
-                                                              fmaf(h.al.x, p.x, -h.al.y * p.y))))),
-          fmaf(h.ah.x, p.y, fmaf(h.ah.y, p.x, fmaf(bc.x, o.y, fmaf(bc.y, o.x,
-                                                             fmaf(h.al.x, p.y, h.al.y * p.x))))));
+      v[i] = half_cell(v[i], o, cc[i], h, env);
     }
   }
 
@@ -237,8 +214,8 @@ struct Quad {
       for (int s = 0; s < kSets; ++s)
         c.tab[s][i] = __ldg(gtab + size_t(s) * 2 * N + (p % 16) * T + p / 16);
     }
-    const Half h0 = half(A.coef[size_t(ch) * kSets], env);
-    const Half h1 = half(A.coef[size_t(ch) * kSets + kSets - 1], env);
+    const HalfCoef h0 = half_coef(A.coef[size_t(ch) * kSets], env);
+    const HalfCoef h1 = half_coef(A.coef[size_t(ch) * kSets + kSets - 1], env);
     float2* field = (env ? A.eh : A.e0) + size_t(ch) * N;
     float2 v[4];
 #pragma unroll
