@@ -229,8 +229,9 @@ BPM_API bpm_status bpm_get_stats(bpm_plan plan, bpm_stats* out);
  *
  *   form               2D march: 0 = propagator tables in shared memory and
  *                      twiddles in registers, one channel group per SM (with
- *                      channels_per_block = 1 and few channels, Nx <= 1024: a
- *                      channel spread over 8 Nx/16 threads);
+ *                      channels_per_block = 1 and few channels: a channel
+ *                      spread over 8 Nx/16 threads at Nx <= 1024, over 2 Nx/16,
+ *                      an envelope each half, at Nx = 2048);
  *                      1 = tables and twiddles read from L2, at most 128
  *                      registers, two channel groups per SM (first order,
  *                      Nx <= 4096, channels_per_block = the size's maximum);
