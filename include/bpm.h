@@ -357,7 +357,10 @@ BPM_API bpm_status bpm_batch_run(bpm_batch b);
  * deformation factor, tables and incident field from the inputs stored by
  * bpm_set_crystal / bpm_set_pulse (device pointers must still be valid), one
  * round to nz and the time responses.  Captured on first use and whenever the
- * set of plans changes, replayed otherwise.  Asynchronous. */
+ * set of plans, their crystals, beams, shards or the batch's cap have changed,
+ * replayed otherwise.  Asynchronous.
+ * Errors: STATE (a crystal set after the pulse that the pulse does not go with),
+ * OOM, CUDA. */
 BPM_API bpm_status bpm_batch_run_graph(bpm_batch b);
 
 /* Kernel launches in one replay of the graph bpm_batch_run_graph captured

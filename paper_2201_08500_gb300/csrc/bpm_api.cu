@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -222,6 +223,7 @@ bool device_ready(int* sm_count) {
 }  // namespace bpm
 
 struct bpm_plan_s {
+  uint64_t id = 0;  // no two plans of a process have the same
   bpm_grid grid{};
   int n_ch = 0;
   cudaStream_t stream = nullptr;
@@ -253,7 +255,7 @@ struct bpm_plan_s {
   // one copy each way: weights and then frequencies, R and then T
   double2* weight = nullptr;
   double* omega = nullptr;
-  std::vector<double> pulse_host;  // the same, gathered for the copy
+  std::vector<double> pulse_host;  // the same of the last pulse, gathered for the copy
   double* inc_norm = nullptr;
   double* refl = nullptr;
   double* trans = nullptr;
@@ -417,6 +419,37 @@ cudaError_t enqueue_crystal(bpm_plan p) {
   return launch_deformation(p->sa, p->u_dev, p->cfield, p->cspan, p->ext, p->stream);
 }
 
+// Whether the channels' frequencies go with the plan's grid and crystal.
+bpm_status check_omega(bpm_plan p, const double* omega) {
+  for (int i = 0; i < p->n_ch; ++i)
+    if (!(omega[i] > 0.0)) return fail(p, BPM_ERR_INVALID_ARG, "omega must be positive");
+  for (int i = 0; i < p->n_ch; ++i)
+    if (!(omega[i] / 299792458.0 > 0.5 * p->sa.h))
+      return fail(p, BPM_ERR_INVALID_ARG, "a channel has k <= h/2 (no Bragg solution)");
+  if (p->grid.split_order == 4) {
+    // the propagation 1-2t < 0 runs backwards: an evanescent mode would grow by
+    // exp((2t-1) dz kappa) before the forward steps damp it; require every
+    // mode of the grid to propagate, |q| + h/2 < k
+    const double qmax = kPiHost / p->grid.dx + 0.5 * p->sa.h;
+    for (int i = 0; i < p->n_ch; ++i)
+      if (!(omega[i] / 299792458.0 > qmax))
+        return fail(p, BPM_ERR_UNSUPPORTED, "fourth-order splitting needs propagating modes only");
+  }
+  if (p->grid.dims == 3) {
+    // the column pass expands sqrt(K^2 - qy^2) - K to second order in
+    // c = dz qy^2 / (2K): require every K^2 > 0 and c < 1e-3 (terms dropped < 2e-10)
+    const double qxm = kPiHost / p->grid.dx + 0.5 * p->sa.h;
+    const double qym = kPiHost / p->grid.dy;
+    for (int i = 0; i < p->n_ch; ++i) {
+      const double k = omega[i] / 299792458.0;
+      const double K2 = k * k - qxm * qxm;
+      if (!(K2 > 0.0) || p->grid.dz * qym * qym / (2.0 * std::sqrt(K2)) > 1e-3)
+        return fail(p, BPM_ERR_UNSUPPORTED, "3D grid too fine for the paraxial y correction");
+    }
+  }
+  return BPM_OK;
+}
+
 // Tables, coefficients and incident field from the stored pulse; march back to z = 0.
 cudaError_t enqueue_pulse(bpm_plan p) {
   cudaError_t e = p->grid.dims == 3
@@ -474,6 +507,8 @@ BPM_API bpm_status bpm_plan_create(const bpm_grid* grid, int n_channels, void* c
     return fail(nullptr, BPM_ERR_UNSUPPORTED, "libbpm is built for sm_103a (GB300) only");
 
   auto p = std::make_unique<bpm_plan_s>();
+  static std::atomic<uint64_t> last_id{0};
+  p->id = ++last_id;
   p->grid = g;
   p->n_ch = n_channels;
   p->stream = static_cast<cudaStream_t>(cuda_stream);
@@ -697,32 +732,7 @@ BPM_API bpm_status bpm_set_pulse(bpm_plan p, const double* omega, const double* 
   if (!omega || !weight_re_im) return fail(p, BPM_ERR_INVALID_ARG, "null omega or weights");
   if (!p->have_crystal) return fail(p, BPM_ERR_STATE, "bpm_set_crystal must come first");
   if (!(w0 > 0.0)) return fail(p, BPM_ERR_INVALID_ARG, "w0 must be positive");
-  for (int i = 0; i < p->n_ch; ++i)
-    if (!(omega[i] > 0.0)) return fail(p, BPM_ERR_INVALID_ARG, "omega must be positive");
-  for (int i = 0; i < p->n_ch; ++i)
-    if (!(omega[i] / 299792458.0 > 0.5 * p->sa.h))
-      return fail(p, BPM_ERR_INVALID_ARG, "a channel has k <= h/2 (no Bragg solution)");
-  if (p->grid.split_order == 4) {
-    // the propagation 1-2t < 0 runs backwards: an evanescent mode would grow by
-    // exp((2t-1) dz kappa) before the forward steps damp it; require every
-    // mode of the grid to propagate, |q| + h/2 < k
-    const double qmax = kPiHost / p->grid.dx + 0.5 * p->sa.h;
-    for (int i = 0; i < p->n_ch; ++i)
-      if (!(omega[i] / 299792458.0 > qmax))
-        return fail(p, BPM_ERR_UNSUPPORTED, "fourth-order splitting needs propagating modes only");
-  }
-  if (p->grid.dims == 3) {
-    // the column pass expands sqrt(K^2 - qy^2) - K to second order in
-    // c = dz qy^2 / (2K): require every K^2 > 0 and c < 1e-3 (terms dropped < 2e-10)
-    const double qxm = kPiHost / p->grid.dx + 0.5 * p->sa.h;
-    const double qym = kPiHost / p->grid.dy;
-    for (int i = 0; i < p->n_ch; ++i) {
-      const double k = omega[i] / 299792458.0;
-      const double K2 = k * k - qxm * qxm;
-      if (!(K2 > 0.0) || p->grid.dz * qym * qym / (2.0 * std::sqrt(K2)) > 1e-3)
-        return fail(p, BPM_ERR_UNSUPPORTED, "3D grid too fine for the paraxial y correction");
-    }
-  }
+  if (const bpm_status st = check_omega(p, omega); st != BPM_OK) return st;
   p->sa.theta_i = theta_i;
   p->sa.x0 = x0;
   p->sa.w0 = w0;
@@ -732,11 +742,11 @@ BPM_API bpm_status bpm_set_pulse(bpm_plan p, const double* omega, const double* 
   const size_t n = size_t(p->n_ch);
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   BPM_CUDA(p, cudaStreamIsCapturing(p->stream, &capture), "upload pulse");
+  p->pulse_host.resize(3 * n);
+  std::memcpy(p->pulse_host.data(), weight_re_im, 2 * n * sizeof(double));
+  std::memcpy(p->pulse_host.data() + 2 * n, omega, n * sizeof(double));
   if (capture == cudaStreamCaptureStatusNone) {
     // one copy from pageable memory, which it has left when the call returns
-    p->pulse_host.resize(3 * n);
-    std::memcpy(p->pulse_host.data(), weight_re_im, 2 * n * sizeof(double));
-    std::memcpy(p->pulse_host.data() + 2 * n, omega, n * sizeof(double));
     BPM_CUDA(p, cudaMemcpyAsync(p->weight, p->pulse_host.data(), 3 * n * sizeof(double),
                                 cudaMemcpyHostToDevice, p->stream),
              "upload pulse");
@@ -1267,7 +1277,7 @@ struct bpm_batch_s {
   int next_slot = 0;
   RoundSlot graph_slot;
   cudaGraphExec_t graph = nullptr;
-  uint64_t graph_key = 0;
+  std::vector<uint64_t> graph_key;
   std::string err = "no error";
   int rounds = 0;
   int last_items[2] = {0, 0};
@@ -1346,6 +1356,35 @@ MarchArgs march_args(bpm_plan p, int n_steps) {
   a.n_steps = n_steps;
   a.split_order = p->grid.split_order;
   return a;
+}
+
+// What the launches of a captured pass hold by value (the rest they read from the
+// plans' buffers): the plans, their inputs and buffers that may be exchanged, and
+// the cap.
+std::vector<uint64_t> graph_values(bpm_batch b) {
+  std::vector<uint64_t> key{uint64_t(b->max_blocks)};
+  auto mix = [&key](auto... v) {
+    for (double d : {double(v)...}) {
+      uint64_t bits;
+      std::memcpy(&bits, &d, sizeof bits);
+      key.push_back(bits);
+    }
+  };
+  auto mix_ptr = [&key](const void* q) { key.push_back(reinterpret_cast<uintptr_t>(q)); };
+  for (const auto& e : b->entries) {
+    const bpm_plan p = e.plan;
+    const SetupArgs& a = p->sa;
+    key.push_back(p->id);
+    // (grid, channel count, order and zassenhaus are the plan's for good)
+    mix(a.h, a.chi0_re, a.chi0_im, a.chih_re, a.chih_im, a.chihb_re, a.chihb_im, a.x_surface,
+        a.x_end, a.tan_psi, a.z_begin, a.z_end, a.theta_i, a.x0, a.w0, a.zx, a.zR);
+    mix(p->domega, p->shard_first, time_rows(p));
+    mix_ptr(a.mask);
+    mix_ptr(p->u_dev);
+    mix_ptr(p->eh_time);
+    mix_ptr(p->time_tab);
+  }
+  return key;
 }
 
 // Enqueue one round on b->stream using slot r: every active entry advances
@@ -1583,20 +1622,17 @@ BPM_API bpm_status bpm_batch_sync(bpm_batch b) {
 // Replays, as one CUDA graph, the whole hot path of every entry in the batch:
 // deformation factor, tables and incident field from the stored inputs, one
 // round to nz, time response.  The graph is captured on the first call and
-// again whenever the set of entries changes.
+// again whenever the set of entries or a value that the launches hold changes.
 BPM_API bpm_status bpm_batch_run_graph(bpm_batch b) {
   BPM_NVTX();
   if (!b) return bfail(nullptr, BPM_ERR_INVALID_ARG, "null batch");
-  uint64_t key = 1469598103934665603ull;
-  auto mix = [&key](uint64_t v) { key = (key ^ v) * 1099511628211ull; };
-  for (const auto& e : b->entries) {
-    mix(reinterpret_cast<uintptr_t>(e.plan));
-    // a shard declared since the capture has other time-response buffers
-    mix(reinterpret_cast<uintptr_t>(e.plan->eh_time));
-    mix(reinterpret_cast<uintptr_t>(e.plan->time_tab));
-    mix(uint64_t(e.plan->shard_first) << 32 | uint32_t(time_rows(e.plan)));
-  }
+  std::vector<uint64_t> key = graph_values(b);
   if (!b->graph || key != b->graph_key) {
+    // a crystal set after the pulse: the stored pulse has to go with it
+    for (const auto& e : b->entries)
+      if (!e.plan->have_pulse &&
+          check_omega(e.plan, e.plan->pulse_host.data() + 2 * size_t(e.plan->n_ch)) != BPM_OK)
+        return bfail(b, BPM_ERR_STATE, "stored pulse and new crystal: " + e.plan->err);
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
     BPM_BCUDA(b, cudaStreamSynchronize(b->stream), "pre-capture sync");
@@ -1650,7 +1686,7 @@ BPM_API bpm_status bpm_batch_run_graph(bpm_batch b) {
     cudaError_t ie = cudaGraphInstantiate(&b->graph, g, 0);
     cudaGraphDestroy(g);
     BPM_BCUDA(b, ie, "graph instantiate");
-    b->graph_key = key;
+    b->graph_key = std::move(key);
     b->graph_slot.used = false;  // the captured round has not run yet
   }
   for (auto& e : b->entries) {
