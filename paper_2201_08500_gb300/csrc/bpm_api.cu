@@ -356,8 +356,8 @@ bool launch_valid(const bpm_grid& g, int form, int group, int row_threads) {
   const int maxg = march_max_group(g.nx);
   if (row_threads != 256) return false;
   if (form == 0) return group == 1 || group == maxg;
-  if (form == 3 && g.nx == 1024)  // two channels per block, first order
-    return group == march_parked_group(g.nx, form) && g.split_order == 1;
+  if (form == 3 && g.nx == 1024)  // two channels per block, first order and Strang
+    return group == march_parked_group(g.nx, form) && g.split_order <= 2;
   if (form == 2 || form == 3)
     return group == 1 &&
            (g.split_order == 1 || (form == 3 && g.split_order == 2) ||

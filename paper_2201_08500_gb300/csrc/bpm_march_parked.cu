@@ -1,9 +1,9 @@
-// First-order resident march, parked forms (Parked<N>: one envelope in
+// Resident march, parked forms (Parked<N>: one envelope in
 // registers, the other in shared memory, at most 128 registers): one channel
 // per block of N/16 threads and 512/(N/16) blocks per SM, each at its own FFT
 // phase.  Form 2 (Nx = 1024, 2048, 4096, first or fourth order) reads the
-// tables from L2; form 3 (Nx = 2048, 4096, 8192, first order or Strang) keeps
-// them in tensor memory (Nx = 1024, first order: two channels per block).
+// tables from L2; form 3 (Nx = 1024 ... 8192, first order or Strang) keeps them in
+// tensor memory (at Nx = 1024 two channels per block).
 // Same per-channel arithmetic as the other forms (bitwise the same fields).
 #include <cuda_runtime.h>
 
