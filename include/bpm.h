@@ -258,7 +258,8 @@ BPM_API bpm_status bpm_get_stats(bpm_plan plan, bpm_stats* out);
  *                      see above), i.e. a tile
  *                      of 256/T or 512/T rows (T = nx/16); taller tiles move
  *                      longer column segments in the transposed store.
- *   ms                 bpm_tune: median time of `steps` steps in this form. */
+ *   ms                 bpm_tune: time of `steps` steps in this form (the median run's
+ *                      share, if the run was longer). */
 typedef struct {
   int32_t form;
   int32_t channels_per_block;
@@ -284,8 +285,8 @@ BPM_API bpm_status bpm_set_launch(bpm_plan plan, const bpm_launch* form);
  * plans of the same (dims, nx, ny, split_order, n_channels) in this process.
  * best receives the fastest; all (capacity max_all, may be NULL) receives every
  * measured form, and n_all their count.  Runs on its own stream and waits for it.
- * Use a few hundred steps: short runs over-weight one-time costs (the
- * shared-memory form copies each channel's tables once per launch).
+ * 2D runs of fewer than 48 steps are lengthened to 48: short ones over-weight
+ * one-time costs (a form copies each channel's tables once per launch).
  * Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
 BPM_API bpm_status bpm_tune(const bpm_grid* grid, int n_channels, int steps, bpm_launch* best,
                             bpm_launch* all, int max_all, int* n_all);

@@ -1059,6 +1059,14 @@ std::string device_tag() {
   return name + "/" + std::to_string(prop.multiProcessorCount);
 }
 
+// A form's one-time costs (tables copied or put into tensor memory, what equal shares
+// march more) are those of a few steps, so the tuner lengthens a shorter 2D run: at 16
+// steps it named forms that a long march is slower in than in the plan's own, at 48
+// the same ones (us a step, tuned in 16 steps against untuned: 330 channels of 1024
+// points, Strang, 5.56 against 4.64; 400 of 1024 4.36 against 3.81; 400 of 2048 7.46
+// against 6.61).
+constexpr int kTuneSteps = 48;
+
 // Times `steps` steps of plan p in its current form: one warm-up, median of three.
 bpm_status time_form(bpm_plan p, int steps, cudaEvent_t e0, cudaEvent_t e1, float* ms) {
   float t[3];
@@ -1083,8 +1091,9 @@ BPM_API bpm_status bpm_tune(const bpm_grid* grid, int n_channels, int steps, bpm
   BPM_NVTX();
   if (!grid || !best || n_channels < 1 || steps < 1 || (all && max_all < 0))
     return fail(nullptr, BPM_ERR_INVALID_ARG, "bpm_tune: bad arguments");
+  const int n = grid->dims == 2 ? std::max(steps, kTuneSteps) : steps;
   bpm_grid g = *grid;
-  g.nz = steps;
+  g.nz = n;
   cudaStream_t s = nullptr;
   if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess)
     return fail(nullptr, BPM_ERR_CUDA, "bpm_tune: stream");
@@ -1130,7 +1139,8 @@ BPM_API bpm_status bpm_tune(const bpm_grid* grid, int n_channels, int steps, bpm
     }
     for (size_t i = 0; st == BPM_OK && i < cand.size(); ++i) {
       st = bpm_set_launch(p, &cand[i]);
-      if (st == BPM_OK) st = time_form(p, steps, e0, e1, &cand[i].ms);
+      if (st == BPM_OK) st = time_form(p, n, e0, e1, &cand[i].ms);
+      cand[i].ms *= float(steps) / float(n);
       if (st == BPM_OK) meas.push_back(cand[i]);
     }
   }

@@ -71,3 +71,11 @@ def test_strang_takes_the_two_channel_form_from_a_caller_and_a_file(tmp_path):
     for got in out[1:]:
         for a, b in zip(out[0], got):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n_ch", [400, 512, 700])
+def test_a_few_tuning_steps_name_the_form_of_a_long_march(n_ch):
+    """Where a form's one-time costs decided in 16 steps: what the tuner names then is what
+    it names in 300 (the forms are 4 % apart or more in the lengthened run)."""
+    named = [bpm.tune(2, 2048, 1, 5e-7, 0.0, 5e-7, n_ch, steps=s)[0] for s in (16, 300)]
+    assert {k: named[0][k] for k in FORM} == {k: named[1][k] for k in FORM}
