@@ -1255,6 +1255,7 @@ struct BatchEntry {
   bpm_plan plan = nullptr;
   cudaStream_t orig_stream = nullptr;  // restored when the ticket completes or is cancelled
   uint64_t ticket = 0;
+  size_t bytes = 0;        // its share of the budget: the plan's bytes when it was admitted
   bool finishing = false;  // finalize enqueued, done event recorded
   bool cancelled = false;
   cudaEvent_t done = nullptr;
@@ -1554,9 +1555,10 @@ BPM_API bpm_status bpm_batch_submit(bpm_batch b, bpm_plan p, uint64_t* ticket) {
     p->stream = b->stream;
   }
   e.plan = p;
+  e.bytes = p->bytes;
   e.ticket = b->next_ticket++;
   b->entries.push_back(e);
-  b->used += p->bytes;
+  b->used += e.bytes;
   *ticket = e.ticket;
   return BPM_OK;
 }
@@ -1593,7 +1595,7 @@ BPM_API bpm_status bpm_batch_poll(bpm_batch b, uint64_t ticket, int* done) {
     e.done = nullptr;
     // no round enqueued after the completing one touches this plan
     e.plan->stream = e.orig_stream;
-    b->used -= e.plan->bytes;
+    b->used -= e.bytes;
     b->finished[ticket] = 1;
     b->entries.erase(b->entries.begin() + long(i));
     *done = 1;
@@ -1614,7 +1616,7 @@ BPM_API bpm_status bpm_batch_cancel(bpm_batch b, uint64_t ticket) {
     if (b->side) BPM_BCUDA(b, cudaStreamSynchronize(b->side), "cancel");
     e.plan->stream = e.orig_stream;
     if (e.done) cudaEventDestroy(e.done);
-    b->used -= e.plan->bytes;
+    b->used -= e.bytes;
     b->finished[ticket] = 2;
     b->entries.erase(b->entries.begin() + long(i));
     return BPM_OK;
