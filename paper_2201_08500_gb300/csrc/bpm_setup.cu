@@ -437,8 +437,13 @@ __device__ __forceinline__ float log_gauss(const SetupArgs& sa, dc inv_den) {
   return -float(inv_den.re / (sa.w0 * sa.w0));
 }
 constexpr float kLogZero = -106.f;
-// |g|^2 below e^-760 is zero in FP64
-constexpr float kLogNormZero = -380.f;
+// |g|^2 below e^-760 is zero in FP64, g below e^-750
+constexpr float kLogNormZero = -380.f, kLogGaussZero = -750.f;
+// A grid that lies wholly where |g| < e^-200 (a beam 14 waists off its edge): the norm's
+// sum is of |kFarScale g|^2, so that |S g|^2 of any S is found where |g|^2 alone would be
+// lost.
+constexpr float kLogFar = -200.f;
+constexpr double kFarScale = 0x1p600;
 
 // Constants of a block's channels, one lane of the first warp each; below the
 // log|g| `least` no channel's value is above zero (-inf with a NaN amplitude).
@@ -447,7 +452,8 @@ struct IncChannels {
   dc sp[kIncMaxCh];
   double dq[kIncMaxCh];
   float bound[kIncMaxCh];
-  float least;
+  float least, norm_zero, log_g;  // log_g: log_gauss
+  bool far;
 };
 __device__ void load_channels(const SetupArgs& sa, const double* omega, const double2* weight,
                               int ch0, int nch, IncChannels* s) {
@@ -468,15 +474,24 @@ __device__ void load_channels(const SetupArgs& sa, const double* omega, const do
       least = l == l ? fminf(least, l) : -INFINITY;  // stays: fminf(-inf, l)
     }
     s->least = least;
+    const double last = double(sa.nx - 1) * sa.dx;
+    const double d = sa.x0 < 0.0 ? sa.x0 : sa.x0 > last ? sa.x0 - last : 0.0;
+    s->log_g = log_gauss(sa, s->beam.inv_den);
+    s->far = s->log_g * float(d * d) < kLogFar;
+    s->norm_zero = s->far ? kLogGaussZero : kLogNormZero;
   }
   __syncthreads();
+}
+__device__ __forceinline__ double norm_part(dc g, bool far) {
+  if (far) g = dscale(g, kFarScale);
+  return g.re * g.re + g.im * g.im;
 }
 
 // The last of `blocks` blocks to leave their parts of the sum of |g|^2 adds the
 // `parts` parts, in an order that depends on their number alone, and writes every
 // channel's norm.
-__device__ void finish_norm(const SetupArgs& sa, const double2* weight, dc pref, int blocks,
-                            int parts, NormScratch* scratch, double* inc_norm) {
+__device__ void finish_norm(const SetupArgs& sa, const double2* weight, dc pref, bool far,
+                            int blocks, int parts, NormScratch* scratch, double* inc_norm) {
   __shared__ int last;
   __shared__ double total;
   __syncthreads();
@@ -499,7 +514,12 @@ __device__ void finish_norm(const SetupArgs& sa, const double2* weight, dc pref,
   __syncthreads();
   for (int c = threadIdx.x; c < sa.n_ch; c += blockDim.x) {
     const dc sp = amplitude(pref, weight[c]);
-    inc_norm[c] = (sp.re * sp.re + sp.im * sp.im) * total;
+    double norm = (sp.re * sp.re + sp.im * sp.im) * total;
+    if (far) {
+      const double m = hypot(sp.re, sp.im) * sqrt(total) / kFarScale;
+      norm = m * m;
+    }
+    inc_norm[c] = norm;
   }
 }
 
@@ -520,9 +540,9 @@ __global__ void __launch_bounds__(THREADS)
   load_channels(sa, omega, weight, ch0, nch, &sc);
   const dc inv_den = sc.beam.inv_den;
   const double x = double(j) * sa.dx, d = x - sa.x0, r2 = d * d;
-  const float lg = log_gauss(sa, inv_den) * float(r2);
+  const float lg = sc.log_g * float(r2);
   dc g = dmk(0.0, 0.0);
-  if (!(lg < (ch0 == 0 ? fminf(sc.least, kLogNormZero) : sc.least))) g = gauss(sa, inv_den, r2);
+  if (!(lg < (ch0 == 0 ? fminf(sc.least, sc.norm_zero) : sc.least))) g = gauss(sa, inv_den, r2);
   for (int c = 0; c < nch; ++c) {
     float2 v = make_float2(0.f, 0.f);
     if (!(lg < kLogZero - sc.bound[c])) {
@@ -535,10 +555,10 @@ __global__ void __launch_bounds__(THREADS)
     eh[size_t(ch0 + c) * sa.nx + j] = make_float2(0.f, 0.f);
   }
   if (ch0 == 0) {
-    double part = g.re * g.re + g.im * g.im;
+    double part = norm_part(g, sc.far);
     for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, off);
     if (threadIdx.x % 32 == 0) scratch->part[j / 32] = part;
-    finish_norm(sa, weight, sc.beam.pref, chunks, sa.nx / 32, scratch, inc_norm);
+    finish_norm(sa, weight, sc.beam.pref, sc.far, chunks, sa.nx / 32, scratch, inc_norm);
   }
   after_tables();
 }
@@ -564,8 +584,8 @@ __global__ void __launch_bounds__(kIncThreads)
   const size_t plane = size_t(sa.nx) * sa.ny;
   // two neighbouring cells a thread: 32 threads a row of the tile
   const int jj = 2 * (threadIdx.x % (kIncTile / 2));
-  const float lgs = log_gauss(sa, sc.beam.inv_den);
-  const float least = ch0 == 0 ? fminf(sc.least, kLogNormZero) : sc.least;
+  const float lgs = sc.log_g;
+  const float least = ch0 == 0 ? fminf(sc.least, sc.norm_zero) : sc.least;
   // no cell of the tile is nearer to the beam's centre than this, and rounding
   // keeps the order
   auto nearest = [](double lo, double hi, double at) {
@@ -583,7 +603,7 @@ __global__ void __launch_bounds__(kIncThreads)
       }
     if (ch0 == 0) {
       if (threadIdx.x == 0) scratch->part[tile] = 0.0;
-      finish_norm(sa, weight, sc.beam.pref, tiles, tiles, scratch, inc_norm);
+      finish_norm(sa, weight, sc.beam.pref, sc.far, tiles, tiles, scratch, inc_norm);
     }
     after_tables();
     return;
@@ -608,7 +628,7 @@ __global__ void __launch_bounds__(kIncThreads)
       lg[h] = lgs * float(r2);
       g[h] = dmk(0.0, 0.0);
       if (!(lg[h] < least)) g[h] = gauss(sa, inv_den, r2);
-      acc += g[h].re * g[h].re + g[h].im * g[h].im;
+      acc += norm_part(g[h], sc.far);
     }
     for (int c = 0; c < nch; ++c) {
       float2 v[2];
@@ -633,7 +653,7 @@ __global__ void __launch_bounds__(kIncThreads)
       for (int w = 1; w < kIncThreads / 32; ++w) acc += red[w];
       scratch->part[tile] = acc;
     }
-    finish_norm(sa, weight, sc.beam.pref, tiles, tiles, scratch, inc_norm);
+    finish_norm(sa, weight, sc.beam.pref, sc.far, tiles, tiles, scratch, inc_norm);
   }
   after_tables();
 }
