@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include "bpm_fft.cuh"
+#include "bpm_half.cuh"
 #include "bpm_internal.h"
 #include "bpm_tma.cuh"
 
@@ -292,32 +293,6 @@ __global__ void __launch_bounds__(ColStream<NY>::kBlock, ColStream<NY>::kBlocksP
   }
 }
 
-// Coupling of one envelope's value with the other's (couple3d's operations):
-// own <- a own + b c' other, c' = c for E0 and conj(c) for Eh.
-struct HalfCoef {
-  float2 ah, al;
-  float bx, r1, py, r2;
-};
-BPM_DEV HalfCoef half_coef(const ChannelCoef& cf, int env) {
-  const float2 b = env ? cf.bm : cf.bp;
-  HalfCoef h;
-  h.ah = cf.a_hi;
-  h.al = cf.a_lo;
-  h.bx = b.x;
-  h.r1 = env ? b.y : -b.y;
-  h.py = env ? b.y : b.x;
-  h.r2 = env ? -b.x : b.y;
-  return h;
-}
-BPM_DEV float2 couple_half(float2 p, float2 o, float2 c, const HalfCoef& h, int env) {
-  const float2 bc = make_float2(fmaf(h.bx, c.x, h.r1 * c.y),
-                                fmaf(h.py, env ? c.x : c.y, h.r2 * (env ? c.y : c.x)));
-  return make_float2(
-      fmaf(h.ah.x, p.x, fmaf(-h.ah.y, p.y, fmaf(bc.x, o.x, fmaf(-bc.y, o.y,
-                                                          fmaf(h.al.x, p.x, -h.al.y * p.y))))),
-      fmaf(h.ah.x, p.y, fmaf(h.ah.y, p.x, fmaf(bc.x, o.y, fmaf(bc.y, o.x,
-                                                         fmaf(h.al.x, p.y, h.al.y * p.x))))));
-}
 BPM_DEV float2 shfl2(float2 v, int src) {
   return make_float2(__shfl_sync(0xFFFFFFFFu, v.x, src), __shfl_sync(0xFFFFFFFFu, v.y, src));
 }
@@ -445,7 +420,7 @@ __global__ void __launch_bounds__(RowStream<NX, R>::kBlock, RowStream<NX, R>::kB
         for (int h = 0; h < F::H; ++h) {
           const float2 c = F::H == 2 ? shfl2(cv[k], (lane & ~1) | h) : cv[k];
           const float2 o = shfl2(v[h][k], lane ^ 1);
-          if (c.x != 0.f || c.y != 0.f) v[h][k] = couple_half(v[h][k], o, c, hc, env);
+          if (c.x != 0.f || c.y != 0.f) v[h][k] = half_cell(v[h][k], o, c, hc, env);
         }
       }
     }

@@ -1,9 +1,10 @@
 // One envelope's half of the coupling, for marches that hold the envelopes in
 // different threads: own <- a own + b c' other, c' = c for E0 (env 0) and conj(c) for
-// Eh, in couple_cell's operations.
+// Eh, in the operations of couple_cell and couple3d.
 #pragma once
 
-#include "bpm_resident.cuh"
+#include "bpm_fft.cuh"
+#include "bpm_internal.h"
 
 namespace bpm {
 
