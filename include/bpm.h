@@ -343,9 +343,9 @@ BPM_API bpm_status bpm_batch_create(size_t hbm_budget_bytes, void* cuda_stream, 
 BPM_API bpm_status bpm_batch_submit(bpm_batch b, bpm_plan plan, uint64_t* ticket);
 
 /* Enqueues one round: every admitted, unfinished plan advances
- * min(chunk_steps, nz - z) steps in one persistent launch (plus a sibling
- * launch for Nx = 8192 on a forked stream); plans that reach nz then get their
- * reflectivity and time response and a completion event.  Asynchronous.
+ * min(chunk_steps, nz - z) steps in one persistent launch per queue (plans of one
+ * size and order); plans that reach nz then get their reflectivity and time
+ * response and a completion event.  Asynchronous.
  * Plans admitted after this call join the next round (continuous batching).
  * Errors: INVALID_ARG, CUDA. */
 BPM_API bpm_status bpm_batch_step(bpm_batch b, int chunk_steps);

@@ -1247,7 +1247,7 @@ BPM_API void bpm_plan_destroy(bpm_plan p) {
 }  // extern "C"
 
 // ===========================================================================
-// Batches: many plans marched by one persistent work-queue launch per round.
+// Batches: many plans marched by persistent work-queue launches, one a queue and round.
 // ===========================================================================
 namespace {
 
@@ -1277,9 +1277,7 @@ struct RoundSlot {
 
 struct bpm_batch_s {
   cudaStream_t stream = nullptr;
-  cudaStream_t side = nullptr;  // Nx = 8192 kernel runs here, forked from stream
   cudaStream_t cap = nullptr;   // graph capture stream (the caller's may be the legacy stream)
-  cudaEvent_t fork = nullptr, join = nullptr;
   size_t budget = 0, used = 0;
   uint64_t next_ticket = 1;
   std::vector<BatchEntry> entries;
@@ -1526,10 +1524,7 @@ BPM_API bpm_status bpm_batch_create(size_t hbm_budget_bytes, void* cuda_stream, 
   auto b = std::make_unique<bpm_batch_s>();
   b->stream = static_cast<cudaStream_t>(cuda_stream);
   b->budget = hbm_budget_bytes;
-  BPM_BCUDA(b.get(), cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking), "side stream");
   BPM_BCUDA(b.get(), cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking), "capture stream");
-  BPM_BCUDA(b.get(), cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "event");
-  BPM_BCUDA(b.get(), cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming), "event");
   *out = b.release();
   return BPM_OK;
 }
@@ -1613,7 +1608,6 @@ BPM_API bpm_status bpm_batch_cancel(bpm_batch b, uint64_t ticket) {
     if (e.finishing) return bfail(b, BPM_ERR_STATE, "ticket already finishing");
     // rounds already enqueued may still touch the plan: wait for them
     BPM_BCUDA(b, cudaStreamSynchronize(b->stream), "cancel");
-    if (b->side) BPM_BCUDA(b, cudaStreamSynchronize(b->side), "cancel");
     e.plan->stream = e.orig_stream;
     if (e.done) cudaEventDestroy(e.done);
     b->used -= e.bytes;
@@ -1755,15 +1749,11 @@ BPM_API void bpm_batch_destroy(bpm_batch b) {
   BPM_NVTX();
   if (!b) return;
   cudaStreamSynchronize(b->stream);
-  if (b->side) cudaStreamSynchronize(b->side);
   for (auto& e : b->entries)
     if (e.done) cudaEventDestroy(e.done);
   for (auto& r : b->slots) slot_free(r);
   slot_free(b->graph_slot);
   if (b->graph) cudaGraphExecDestroy(b->graph);
-  if (b->fork) cudaEventDestroy(b->fork);
-  if (b->join) cudaEventDestroy(b->join);
-  if (b->side) cudaStreamDestroy(b->side);
   if (b->cap) cudaStreamDestroy(b->cap);
   delete b;
 }

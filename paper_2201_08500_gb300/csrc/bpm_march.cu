@@ -24,10 +24,6 @@
 
 namespace bpm {
 
-namespace {
-
-}  // namespace
-
 int march_threads_per_channel(int n) { return n / 16; }
 
 int march_max_group(int n) {
