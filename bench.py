@@ -53,34 +53,34 @@ FP32_LANES_PER_SM = 128
 TOL_FIELD = 1e-4
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the
-# default march, from one ncu capture of that launch (form 3 with the packed
-# FP32 butterflies: 555.43 MB read + 55.04 MB written).  The deformation rows
-# are re-read by each wave of channels, which at ~10 GB/s is immaterial to this
-# ALU-bound kernel.  Keyed by kernel, form and workload; any other
+# default march, from one ncu capture of that launch (215.18 MB read + 34.97 MB
+# written: tables and fields, and the deformation rows only inside the crystal;
+# part of the fields stays in L2).  Keyed by kernel, form and workload; any other
 # configuration (or a kernel changed since the capture) reports null.
 MEASURED_TRAFFIC = {
-    ("march_kernel<4096,1> form 3", "deformed-2d-nx4096-nz2000-ch1024", 1): 610.46e6,
+    ("march_kernel<4096,1> form 3", "deformed-2d-nx4096-nz2000-ch1024", 1): 250.15e6,
 }
 # Executed FP32 flop per cell-update (FADD + FMUL + 2 FFMA thread instructions,
 # ncu, per kernel and form): the work the kernel really issues, against the
 # nominal count of flops_per_cell.  Counted on the build with scalar
-# butterfly additions; the packed build performs the same operations (its
-# fields are bitwise equal at these sizes), and ncu's per-opcode FP32 counters
-# do not resolve the packed two-lane instructions.  8192: 240 counted, less
+# butterfly additions; the packed build, and the march whose envelopes take
+# turns, perform the same operations on every element (their fields are
+# bitwise equal), and ncu's per-opcode FP32 counters do not resolve the packed
+# two-lane instructions.  8192: 240 counted, less
 # the products by one that the lane-pair twiddles dropped since (7 complex
 # products of 6 flop per thread, four times a step, over 16 cell-updates).
 EXECUTED_FLOPS = {
     "march_kernel<4096,1> form 3": 210.0,
     "march_kernel<8192,1> form 3": 240.0 - 7 * 6 * 4 / 16,
 }
-# DRAM bytes of one z step of the 3D workload (one streamed column pass, launch
-# form 1, + one MODE-1 row pass, 256-thread row tile), from the live launch
-# list of those launches with --cache-control none: 1066.2 + 1082.6 MB, the
-# algorithmic 64 B per cell-update (2147 MB) within 0.1 %.
+# DRAM bytes of one z step of the 3D workload (column pass read + write, inner row
+# pass read + write; launch form 1 with 256-thread row tiles, form 2 with
+# 128-thread ones), from the live launch list of those launches with
+# --cache-control none: the algorithmic 64 B per cell-update (2147 MB) within 0.2 %.
 MEASURED_TRAFFIC_3D = {("large-3d-512x512-nz1000-ch128", 1, 256): (539.6e6 + 526.6e6 + 537.6e6
                                                                      + 545.0e6),
-                       ("large-3d-512x512-nz1000-ch128", 2, 128): (539.5e6 + 528.3e6 + 538.5e6
-                                                                     + 544.5e6)}
+                       ("large-3d-512x512-nz1000-ch128", 2, 128): (540.1e6 + 528.4e6 + 537.6e6
+                                                                     + 543.3e6)}
 
 
 def flops_per_cell(n: int, split_order: int = 1) -> float:
@@ -400,7 +400,7 @@ def run_batched(args, world, rank, local, jobs=None):
                     f"{max(w.n_ch for w in ws)} channels, perfect / bent / random strain",
         "cell_updates": cells, "l2": "flushed between timed steps (256 MB write)",
         "form": "one CUDA graph: setup of every instance, persistent work-queue launches "
-                "(14 queues by size and splitting order), time responses",
+                "(one per size, splitting order and kind of item), time responses",
         "plain": {"value": cells / (ms_plain * 1e-3), "ms_per_step": ms_plain, "steps": steps_p,
                   "form": "per instance: setup kernels, one march launch in its tuned form, "
                           "time response"},

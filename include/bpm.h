@@ -387,8 +387,8 @@ BPM_API bpm_status bpm_batch_sync(bpm_batch b);
  * Errors: INVALID_ARG, CUDA (a round's kernels failed). */
 BPM_API bpm_status bpm_batch_pending(bpm_batch b, int* rounds_in_flight);
 
-/* Caps the persistent launches of later rounds at max_blocks blocks (one per
- * SM; <= 0 restores every SM).  Two batches on different streams with caps
+/* Caps the persistent launches of later rounds at the blocks that fill max_blocks
+ * SMs (<= 0 restores every SM).  Two batches on different streams with caps
  * that add up to the SM count run side by side, e.g. a lane for short requests
  * next to a lane for long ones.  Errors: INVALID_ARG. */
 BPM_API bpm_status bpm_batch_set_max_blocks(bpm_batch b, int max_blocks);

@@ -6,8 +6,9 @@
 // 1024 one channel in the parked form with tables in tensor memory; below, G =
 // 256 / T channels (T = Nx/16 threads each) of the resident form, and single
 // channels of what fills no such item with 8 T threads (bpm_quad.cuh).  One
-// queue per size, order and kind.  The counter lives in global memory and is
-// cleared before each launch; the queue never waits, so no block can hang.
+// queue per size, order and kind.  The counters live in global memory and are
+// cleared once a round, before its first queue.  No block waits for another's
+// items; block 0 of a queue waits, at its end, for the queue before it.
 #include <cuda_runtime.h>
 
 #include "bpm_parked.cuh"
@@ -79,8 +80,8 @@ using TmBody = Parked<N, SPLIT, true, SPLIT != 1 && N <= 4096>;
 
 // Items at Nx = 2048, 4096, 8192 in the parked form with tables in tensor
 // memory (Parked<N, SPLIT, true>, the fastest single-plan form there): one
-// channel per item, N/16 threads per block, 512/(N/16) blocks per SM; every block allocates its TMEM columns once and
-// frees them on exit.
+// channel per item, N/16 threads per block, 512/(N/16) blocks per SM; every block
+// allocates its TMEM columns once and frees them on exit.
 template <int N, int SPLIT>
 __global__ void __launch_bounds__(N / 16, 512 / (N / 16))
     batch_kernel_tm(const MarchArgs* __restrict__ plans, const BatchItem* __restrict__ items,
@@ -192,8 +193,8 @@ __global__ void __launch_bounds__(Quad<N, SPLIT>::kThreads, 768 / Quad<N, SPLIT>
 // A resident item takes an SM for the time of a full one however few channels
 // it has (us a step, first order, Strang, fourth order: 256 points 2.9, 4.4,
 // 10.3; 512 points 4.7, 5.8, 15.6), a channel of the other form its share of
-// one (0.25, 0.275, 0.85; 0.61, 0.66, 2.31).  One kind for the whole round: the
-// queues run one after the other.
+// one (0.25, 0.275, 0.85; 0.61, 0.66, 2.31).  One kind for all of a round's plans of
+// a size and order: their channels and items are counted together.
 bool batch_singles(int n, int split_order, int channels, int items, int sms) {
   if (n > 512 || sms < 1) return false;
   const int i = n == 256 ? 0 : 1, o = split_order == 1 ? 0 : split_order == 2 ? 1 : 2;

@@ -268,8 +268,8 @@ cudaError_t launch_incident(const SetupArgs& sa, const double* omega, const doub
                             cudaStream_t s);
 
 // Frequency-to-time assembly (bpm_time.cu).  Shape of the transform over n
-// channels: len = n with radices up to 8, or (chirp) the power-of-two length of
-// Bluestein's form.
+// channels: len = n with radices up to 8, or (chirp) the length of Bluestein's form,
+// the cheapest 2^a 3^b 5^c 7^d.
 struct TimeShape {
   int n, len, chirp, n_pass;
   unsigned char radix[16];

@@ -35,8 +35,8 @@
 // begins with the other one.  The coupling touches the parked envelope and the
 // deformation row only where the crystal is (its extent in x over all rows): a
 // Bragg slab fills a tenth of the grid, and the L1 data path, which this march
-// keeps busiest (60 % of its cycles, the FP32 pipe 56 %), carries one park and
-// one unpark a step instead of four passes over an envelope.  Strang adds a
+// keeps busiest (at 4096 points 62 % of its cycles, the FP32 pipe 59 %), carries one
+// park and one unpark a step instead of four passes over an envelope.  Strang adds a
 // coupling before; fourth order runs three (propagate both, couple) rounds
 // after it.  us a step, before and after: 1024 channels of 8192 points 74.8 ->
 // 72.3, 4096 29.9 -> 29.0, 2048 13.85 -> 13.25, 1024 7.65 -> 7.26 (tables in
