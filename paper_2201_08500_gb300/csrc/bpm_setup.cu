@@ -439,9 +439,9 @@ __device__ __forceinline__ float log_gauss(const SetupArgs& sa, dc inv_den) {
 constexpr float kLogZero = -106.f;
 // |g|^2 below e^-760 is zero in FP64, g below e^-750
 constexpr float kLogNormZero = -380.f, kLogGaussZero = -750.f;
-// A grid that lies wholly where |g| < e^-200 (a beam 14 waists off its edge): the norm's
-// sum is of |kFarScale g|^2, so that |S g|^2 of any S is found where |g|^2 alone would be
-// lost.
+// A grid whose cells all have |g| < e^-200 (a beam 14 waists off its edge, or one that
+// falls between two cells): the norm's sum is of |kFarScale g|^2, so that |S g|^2 of any
+// S is found where |g|^2 alone would be lost.
 constexpr float kLogFar = -200.f;
 constexpr double kFarScale = 0x1p600;
 
@@ -474,8 +474,9 @@ __device__ void load_channels(const SetupArgs& sa, const double* omega, const do
       least = l == l ? fminf(least, l) : -INFINITY;  // stays: fminf(-inf, l)
     }
     s->least = least;
-    const double last = double(sa.nx - 1) * sa.dx;
-    const double d = sa.x0 < 0.0 ? sa.x0 : sa.x0 > last ? sa.x0 - last : 0.0;
+    // from the beam's centre to a nearest cell (in 3D there is one at y = 0)
+    const float j = fminf(fmaxf(rintf(float(sa.x0) / float(sa.dx)), 0.f), float(sa.nx - 1));
+    const double d = sa.x0 - double(j) * sa.dx;
     s->log_g = log_gauss(sa, s->beam.inv_den);
     s->far = s->log_g * float(d * d) < kLogFar;
     s->norm_zero = s->far ? kLogGaussZero : kLogNormZero;
